@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
       const int y = row % p.ny, z = row / p.ny;
       constexpr bool SC = scaled_step<P, FO>();
       R d[L::Q];
-      if (interior) pull_interior<L, P, R, LD_RO, SC>(fin + site, p, y, z, d);
+      if (interior) pull_interior<L, P, R, LD_RO, SC ? IN_SCALED : IN_DEV>(fin + site, p, y, z, d);
       else pull<L, P, R, LD_RO, SC>(fin, p, x, y, z, d);
       R g[3];
       site_force_r<L::D, R>(p, x, y, z, site, g);

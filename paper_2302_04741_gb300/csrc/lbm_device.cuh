@@ -320,6 +320,12 @@ __device__ __forceinline__ typename Codec<P>::R step_in(typename Codec<P>::T v, 
   if constexpr (SC) return __half2float(v);
   else return Codec<P>::template decode<L, I>(v, p);
 }
+// the stored value of FP64 storage in the step's arithmetic
+template <int P>
+__device__ __forceinline__ typename Codec<P>::R stored_value(double v) {
+  if constexpr (P == P_FP64DF) return df_split(v);
+  else return v;
+}
 // a deviation formed in the kernel (a wall slot) in the working representation
 template <int I, bool SC, class R>
 __device__ __forceinline__ R step_from_dev(R d, const StepParams& p) {
@@ -573,6 +579,24 @@ __device__ __forceinline__ void rest_terms(const MidState<L, R>& m, R& E, R& Fe)
 // theta is taken from the same f~, so the trace term is dropped.
 // S is stored as (xx, yy, zz, xy, xz, yz); in 2-D the z entries are zero.
 template <class L, class R>
+__device__ __forceinline__ void stress_from_sums(R P0, R P1, R P2, R P3, R P4, R P5, R drho, R rho, R Th,
+                                                 const R (&u)[3], const R (&g)[3], R (&S)[6]) {
+  const R iso = fma(rho, Th, drho);
+  const R hr = R(0.5) * rho;
+  // -rho u_a u_b + rho (u_a g_b + g_a u_b) / 2
+  auto conv = [&](int a, int b) { return hr * (u[a] * (g[b] - u[b]) + u[b] * (g[a] - u[a])); };
+  S[0] = mul_c2<L, R>(P0) - iso + conv(0, 0);
+  S[1] = mul_c2<L, R>(P1) - iso + conv(1, 1);
+  S[3] = mul_c2<L, R>(P3) + conv(0, 1);
+  if constexpr (L::D == 3) {
+    S[2] = mul_c2<L, R>(P2) - iso + conv(2, 2);
+    S[4] = mul_c2<L, R>(P4) + conv(0, 2);
+    S[5] = mul_c2<L, R>(P5) + conv(1, 2);
+  } else {
+    S[2] = S[4] = S[5] = R(0);
+  }
+}
+template <class L, class R>
 __device__ __forceinline__ void stress_tensor(const R (&d)[L::Q], R drho, R rho, R Th,
                                               const R (&u)[3], const R (&g)[3], R (&S)[6]) {
   constexpr int NP = (L::Q - 1) / 2;
@@ -590,20 +614,26 @@ __device__ __forceinline__ void stress_tensor(const R (&d)[L::Q], R drho, R rho,
       P5 = mac<ey * ez>(s, P5);
     }
   });
-  const R iso = fma(rho, Th, drho);
-  const R hr = R(0.5) * rho;
-  // -rho u_a u_b + rho (u_a g_b + g_a u_b) / 2
-  auto conv = [&](int a, int b) { return hr * (u[a] * (g[b] - u[b]) + u[b] * (g[a] - u[a])); };
-  S[0] = mul_c2<L, R>(P0) - iso + conv(0, 0);
-  S[1] = mul_c2<L, R>(P1) - iso + conv(1, 1);
-  S[3] = mul_c2<L, R>(P3) + conv(0, 1);
-  if constexpr (L::D == 3) {
-    S[2] = mul_c2<L, R>(P2) - iso + conv(2, 2);
-    S[4] = mul_c2<L, R>(P4) + conv(0, 2);
-    S[5] = mul_c2<L, R>(P5) + conv(1, 2);
-  } else {
-    S[2] = S[4] = S[5] = R(0);
-  }
+  stress_from_sums<L, R>(P0, P1, P2, P3, P4, P5, drho, rho, Th, u, g, S);
+}
+// the same from the pair sums of the deviations
+template <class L, class R>
+__device__ __forceinline__ void stress_tensor_pairs(const R (&s)[(L::Q - 1) / 2], R drho, R rho, R Th,
+                                                    const R (&u)[3], const R (&g)[3], R (&S)[6]) {
+  R P0 = R(0), P1 = R(0), P2 = R(0), P3 = R(0), P4 = R(0), P5 = R(0);
+  static_for<0, (L::Q - 1) / 2>([&](auto K) {
+    constexpr int k = K, ip = 2 * k + 1;
+    constexpr int ex = L::E(ip, 0), ey = L::E(ip, 1), ez = L::E(ip, 2);
+    P0 = mac<ex * ex>(s[k], P0);
+    P1 = mac<ey * ey>(s[k], P1);
+    P3 = mac<ex * ey>(s[k], P3);
+    if constexpr (L::D == 3) {
+      P2 = mac<ez * ez>(s[k], P2);
+      P4 = mac<ex * ez>(s[k], P4);
+      P5 = mac<ey * ez>(s[k], P5);
+    }
+  });
+  stress_from_sums<L, R>(P0, P1, P2, P3, P4, P5, drho, rho, Th, u, g, S);
 }
 
 // Per-site factors of the odd term k [(g.xi)(xi.S.xi) - 2 (S g).xi] in

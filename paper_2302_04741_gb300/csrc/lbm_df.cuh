@@ -3,8 +3,8 @@
 // GB300 executes FP64 instructions at about 1/73 of the FP32 rate (measured:
 // DFMA and DADD 0.53 T/s, FFMA 38.8 T/s), and its double <-> float
 // conversion instructions run at the FP64 rate too.  The FP64 step (FP64
-// storage, about 620 FP64 operations per site) is therefore bound by the
-// FP64 units at about 1/13 of its HBM roofline.  A value held as an
+// storage, some 440 FP64 operations per site) is therefore bound by the
+// FP64 units at about a tenth of its HBM roofline.  A value held as an
 // unevaluated sum hi + lo of two floats (|lo| <= ulp(hi)) carries about 48
 // significant bits, and its arithmetic -- Dekker's and Knuth's error-free
 // transformations (two-sum, and two-product through the fused multiply-add)
@@ -78,6 +78,11 @@ __device__ __forceinline__ DF operator*(DF a, DF b) {
   e = fmaf(a.lo, b.hi, e);
   return DF(p, e);
 }
+// k * v for a float k that is exact (a small integer): no product with its zero lo
+__device__ __forceinline__ DF df_mulf(float k, DF v) {
+  const float p = __fmul_rn(k, v.hi);
+  return DF(p, fmaf(k, v.lo, fmaf(k, v.hi, -p)));
+}
 // a / b: a float quotient, one correction from the float-float residual
 __device__ __forceinline__ DF operator/(DF a, DF b) {
   df_fast_two_sum(b.hi, b.lo, b.hi, b.lo);
@@ -113,34 +118,38 @@ __device__ __forceinline__ DF fma(DF a, DF b, DF c) {
 
 // The IEEE double d as hi + lo: hi holds the leading 24 significant bits,
 // lo the next 29 bits rounded to 24; built from the bit fields with integer
-// operations.  |d| < 2^-126 gives 0; infinities and NaN go through the
-// conversion instruction (so that an unstable state stays visible).
+// operations and selects (a conversion instruction, even one that only a
+// never-taken case needs, runs at the FP64 rate: three of them per population
+// kept the FP64 unit 55 % busy).  |d| < 2^-126 gives 0; |d| >= 2^128, infinities
+// and NaN give NaN (so that an unstable state stays visible).
 __device__ __forceinline__ DF df_split(double d) {
   const unsigned hi32 = (unsigned)__double2hiint(d), lo32 = (unsigned)__double2loint(d);
   const unsigned E = (hi32 >> 20) & 0x7ffu;  // biased exponent
-  if (E <= 896u) return DF(0.f, 0.f);
-  if (E >= 1139u) return DF((float)d, 0.f);  // |d| >= 2^116 (the lo scale would overflow), inf, NaN
   const unsigned sign = hi32 & 0x80000000u;
   const unsigned m23 = ((hi32 & 0xfffffu) << 3) | (lo32 >> 29);
-  const float hi = __uint_as_float(sign | ((E - 896u) << 23) | m23);
-  // remainder L 2^(E - 1075), L < 2^29, scaled in two exact steps
+  unsigned h = sign | ((E - 896u) << 23) | m23;
+  h = E >= 1151u ? 0x7fc00000u : h;
+  h = E <= 896u ? 0u : h;
+  // remainder L 2^(E - 1075), L < 2^29, scaled in two exact steps; none where
+  // hi is special or the scale would overflow (|d| >= 2^116)
   const float L = (float)(lo32 & 0x1fffffffu);
-  float lo = __fmul_rn(__fmul_rn(L, 0x1p-64f), __uint_as_float((E - 884u) << 23));
-  lo = __uint_as_float(__float_as_uint(lo) | sign);
+  const float lo = __fmul_rn(__fmul_rn(L, 0x1p-64f), __uint_as_float((E - 884u) << 23));
+  const unsigned l = E - 897u < 242u ? (__float_as_uint(lo) | sign) : 0u;
   DF r;
-  df_fast_two_sum(hi, lo, r.hi, r.lo);
+  df_fast_two_sum(__uint_as_float(h), __uint_as_float(l), r.hi, r.lo);
   return r;
 }
 
-// The float f as a double, built bit by bit (exact; zero and float
-// subnormals give 0; inf and NaN through the conversion instruction).
+// The float f as a double, built bit by bit (exact, infinities and NaN too;
+// zero and float subnormals give 0).
 __device__ __forceinline__ double f2d_bits(float f) {
   const unsigned u = __float_as_uint(f);
-  const unsigned e = (u >> 23) & 0xffu;
-  if (e == 0u) return 0.0;
-  if (e == 0xffu) return (double)f;
-  const unsigned hi32 = (u & 0x80000000u) | ((e + 896u) << 20) | ((u & 0x7fffffu) >> 3);
-  return __hiloint2double((int)hi32, (int)(u << 29));
+  const unsigned m = u & 0x7fffffffu;
+  // the exponent moves up by 896, of the special values by twice that
+  unsigned hi32 = (u & 0x80000000u) | ((m >> 3) + (m >= 0x7f800000u ? 1792u << 20 : 896u << 20));
+  hi32 = m < 0x00800000u ? 0u : hi32;
+  const unsigned lo32 = m < 0x00800000u ? 0u : u << 29;
+  return __hiloint2double((int)hi32, (int)lo32);
 }
 
 // hi + lo rounded to the nearest double: one DADD of the exact halves.

@@ -11,6 +11,7 @@
 #pragma once
 
 #include "lbm_device.cuh"
+#include "lbm_poly.cuh"
 
 namespace lbm {
 
@@ -61,6 +62,45 @@ __device__ __forceinline__ void site_force_r(const StepParams& p, int x, int y, 
   if (D == 2) g[2] = R(0);
 }
 
+// What a pull returns per population: the deviation, the scaled value of an
+// FP16-scaled step (see scaled_step), or the stored value itself (FP64 storage:
+// the FP64 steps form pair sums and differences from it, see pair_split).
+enum { IN_DEV = 0, IN_SCALED = 1, IN_STORED = 2 };
+template <class L, int P, int I, int IN>
+__device__ __forceinline__ typename Codec<P>::R pulled_value(typename Codec<P>::T v, const StepParams& p) {
+  if constexpr (IN == IN_STORED) return stored_value<P>(v);
+  else return step_in<L, P, I, IN == IN_SCALED>(v, p);
+}
+
+// Pull of all Q populations of site (x, y, z) of a row that no wall rule
+// touches, with the periodic wrap of every axis.
+template <class L, int P, class RR, int LD = LD_HINT, int IN = IN_DEV>
+__device__ __forceinline__ void pull_wrap(const typename Codec<P>::T* __restrict__ fin,
+                                          const StepParams& p, int x, int y, int z, RR (&d)[L::Q]) {
+  using C = Codec<P>;
+  constexpr int D = L::D, Q = L::Q;
+  const int nx = p.nx, ny = p.ny, nz = p.nz;
+  const size_t N = (size_t)p.N;
+  int xs[7], ys[7], zs[7];
+#pragma unroll
+  for (int k = 0; k < 7; ++k) {
+    xs[k] = wrap3(x - (k - 3), nx);
+    ys[k] = wrap3(y - (k - 3), ny) * nx;
+    zs[k] = D == 3 ? wrap3(z - (k - 3), nz) * nx * ny : 0;
+  }
+  static_for<0, Q>([&](auto I) {
+    constexpr int i = I;
+    constexpr int ex = L::E(i, 0), ey = L::E(i, 1), ez = L::E(i, 2);
+    const int off = zs[ez + 3] + ys[ey + 3] + xs[ex + 3];
+    d[i] = RR(pulled_value<L, P, i, IN>(ldpop<C, LD>(fin + i * N + off, p), p));
+  });
+}
+
+// Whether layer a of the wall axis pulls through a wall rule.
+__device__ __forceinline__ bool near_wall(const StepParams& p, int a, int nA) {
+  return p.wall != W_NONE && (a < 3 || a >= nA - 3);
+}
+
 // Pull of all Q populations of site (x, y, z) with the boundary rules, decoded
 // to deviations in type RR (SC: the scaled values of an FP16-scaled step, see
 // scaled_step).  The wall axis is the last axis (y in 2-D, z in 3-D).
@@ -73,22 +113,16 @@ __device__ __forceinline__ void pull(const typename Codec<P>::T* __restrict__ fi
   const size_t N = (size_t)p.N;
   const int a = D == 2 ? y : z;          // coordinate along the wall axis
   const int nA = D == 2 ? ny : nz;
+  if (!near_wall(p, a, nA)) {
+    pull_wrap<L, P, RR, LD, SC ? IN_SCALED : IN_DEV>(fin, p, x, y, z, d);
+    return;
+  }
   int xs[7], ys[7], zs[7];
 #pragma unroll
   for (int k = 0; k < 7; ++k) {
     xs[k] = wrap3(x - (k - 3), nx);
     ys[k] = wrap3(y - (k - 3), ny) * nx;
     zs[k] = D == 3 ? wrap3(z - (k - 3), nz) * nx * ny : 0;
-  }
-  const bool near = p.wall != W_NONE && (a < 3 || a >= nA - 3);
-  if (!near) {
-    static_for<0, Q>([&](auto I) {
-      constexpr int i = I;
-      constexpr int ex = L::E(i, 0), ey = L::E(i, 1), ez = L::E(i, 2);
-      const int off = zs[ez + 3] + ys[ey + 3] + xs[ex + 3];
-      d[i] = RR(step_in<L, P, i, SC>(ldpop<C, LD>(fin + i * N + off, p), p));
-    });
-    return;
   }
   // ---- a row next to a wall: slots whose source lies beyond the wall
   const int side = a < 3 ? 0 : 1;
@@ -199,7 +233,7 @@ __device__ __forceinline__ void pull_solid(const typename Codec<P>::T* __restric
 // source offset relative to the thread's own site, i*N + (row / plane shift)
 // - e_ix, is the same for the whole block (rows wrap only through the block's
 // y, z), so addresses are a per-thread base plus block-uniform offsets.
-template <class L, int P, class RR, int LD = LD_HINT, bool SC = false>
+template <class L, int P, class RR, int LD = LD_HINT, int IN = IN_DEV>
 __device__ __forceinline__ void pull_interior(const typename Codec<P>::T* __restrict__ fsite,
                                               const StepParams& p, int y, int z,
                                               RR (&d)[L::Q]) {
@@ -216,59 +250,14 @@ __device__ __forceinline__ void pull_interior(const typename Codec<P>::T* __rest
     constexpr int i = I;
     constexpr int ex = L::E(i, 0), ey = L::E(i, 1), ez = L::E(i, 2);
     const long long off = i * N + dz[ez + 3] + dy[ey + 3] - ex;
-    d[i] = RR(step_in<L, P, i, SC>(ldpop<C, LD>(fsite + off, p), p));
+    d[i] = RR(pulled_value<L, P, i, IN>(ldpop<C, LD>(fsite + off, p), p));
   });
 }
 
-// ------------------------------------------ float-float step: pair body
-// The float-float FP64 step executes ~9,700 instructions per site, almost
-// all of it straight-line code: unrolled over the direction pairs it
-// exceeds the instruction cache many times over, and instruction fetch
-// became its top stall.  Its pair body therefore runs out of line, one
-// copy for all pairs, with the pair's directions passed at run time and
-// the site's values in one struct (the arithmetic is the inlined body's,
-// operation for operation, so the results are the same bits): 1.3x faster
-// on GB300.
-struct DFSite {
-  DF cu[3], cs[3], hom1, P4, Q3;
-};
-struct DFPair {
-  DF p, m;
-};
-// k * v and acc + k * v for a small run-time integer k, as imul / mac do
-// for a compile-time one
-__device__ __forceinline__ DF df_imul(int k, DF v) {
-  return k == 0 ? DF() : (k == 1 ? v : (k == -1 ? -v : DF(k) * v));
-}
-__device__ __forceinline__ DF df_mac(int k, DF v, DF acc) {
-  return k == 0 ? acc : (k == 1 ? acc + v : (k == -1 ? acc - v : fma(DF(k), v, acc)));
-}
-template <int D, int FO, bool NEQ4>
-__device__ __noinline__ DFPair df_pair(DF dp, DF dm, int ex, int ey, int ez, DF P0, DF P2, DF Q1, DF A1, DF w,
-                                       const DFSite& S) {
-  DF t = df_imul(ex, S.cu[0]);
-  t = df_mac(ey, S.cu[1], t);
-  if (D == 3) t = df_mac(ez, S.cu[2], t);
-  DF sp = df_imul(ex, S.cs[0]);
-  sp = df_mac(ey, S.cs[1], sp);
-  if (D == 3) sp = df_mac(ez, S.cs[2], sp);
-  const DF t2 = t * t;
-  DF ev_in = fma(t2, NEQ4 ? fma(t2, S.P4, P2) : P2, P0);
-  DF od_in = t * fma(t2, S.Q3, Q1);
-  if (FO >= 1) {
-    ev_in = fma(sp, t, ev_in);
-    od_in = FO >= 2 ? fma(sp, fma(DF(0.5), t2, A1), od_in) : od_in + sp;
-  } else {
-    od_in = od_in + sp;
-  }
-  const DF ev = fma(dp + dm, S.hom1, w * ev_in);
-  const DF od = fma(dp - dm, S.hom1, w * od_in);
-  return DFPair{ev + od, ev - od};
-}
-
 // ------------------------------------------------------------ the step
-// Collision of one site from its pulled deviations d (Eq. lbm) and store of
-// f*(x) at `site`; shared by the plain and the TMA-staged step kernels.
+// Collision of one site from its pulled deviations d (Eq. lbm) in float and
+// store of f*(x) at `site`; shared by all step kernels of the float codecs (FP64
+// storage: poly_store below).
 //
 // f*_i - w_i = d_i (1 - om) + w_i [om drho + rho (om p_i + (1 - om/2) F'_i)],
 // with p_i = E +- O the equilibrium polynomial and F'_i = Fe +- Fo the force
@@ -294,6 +283,7 @@ __device__ __forceinline__ void collide_store(typename Codec<P>::R (&d)[L::Q],
   constexpr int NP = (L::Q - 1) / 2, NS = L::NSHELL, D = L::D;
   constexpr bool EX = P != P_FP16S;  // quadrature constants as hi + lo pairs
   static_assert(!SC || scaled_step<P, FO>(), "scaled values: FP16-scaled storage, FO 0..2");
+  static_assert(std::is_same<R, float>::value, "FP64 storage: poly_store");
   const size_t N = (size_t)p.N;
   const RawMoments<L, R> r = SC ? raw_moments_scaled<L, R>(d, R(p.h_inv_scale)) : raw_moments<L, R>(d);
   // times s: the coefficients of w_i in the scaled representation
@@ -341,9 +331,8 @@ __device__ __forceinline__ void collide_store(typename Codec<P>::R (&d)[L::Q],
   const R base = scl(om * r.drho) - rkgu;
   // rho om multiplies every direction's equilibrium part at this site, so its
   // rounding would act as a common factor (a coherent momentum / energy error
-  // per step): carry it as rom + rom_lo, with the exact FMA residual (in
-  // double the product's rounding is far below the tolerances: rom_lo = 0).
-  const R rom_lo = sizeof(R) == sizeof(double) ? R(0) : scl(fma(rho, om, -rom0));
+  // per step): carry it as rom + rom_lo, with the exact FMA residual.
+  const R rom_lo = scl(fma(rho, om, -rom0));
   static_for<0, NS>([&](auto S) {
     constexpr int sh = S;
     constexpr double X2d = L::c2 * double(L::E2(sh));
@@ -374,36 +363,10 @@ __device__ __forceinline__ void collide_store(typename Codec<P>::R (&d)[L::Q],
   }
   // rest particle: t = s' = 0
   typename C::T* __restrict__ fo = fout + site;
-  // FP64 storage probe: the stored deviation rounded as a float codec stores it
-  const bool probe = P == P_FP64 && p.storage_probe != 0;
-  {
-    R d0 = fma(d[0], om1, SC ? P0[0] : mul_w<L, 0, R, EX>(P0[0]));
-    if constexpr (P == P_FP64)
-      if (probe) d0 = probe_round<0>(d0, p);
-    fo[0] = step_out<L, P, 0, SC>(d0, p);
-  }
-  constexpr bool DF_OUT_OF_LINE = std::is_same<R, DF>::value && FO <= 2;
-  DFSite dfs;
-  if constexpr (DF_OUT_OF_LINE) {
-    for (int a = 0; a < 3; ++a) {
-      dfs.cu[a] = cu[a];
-      dfs.cs[a] = cs[a];
-    }
-    dfs.hom1 = hom1;
-    dfs.P4 = P4;
-    dfs.Q3 = Q3;
-  }
+  fo[0] = step_out<L, P, 0, SC>(fma(d[0], om1, SC ? P0[0] : mul_w<L, 0, R, EX>(P0[0])), p);
   static_for<0, NP>([&](auto K) {
     constexpr int ip = 2 * K + 1, im = ip + 1;
     constexpr int sh = L::SH(ip);
-    if constexpr (DF_OUT_OF_LINE) {
-      constexpr F2 wk = f2_of(L::W(ip));
-      const DFPair o = df_pair<D, FO, (L::NEQ >= 4)>(d[ip], d[im], L::E(ip, 0), L::E(ip, 1), L::E(ip, 2), P0[sh],
-                                                     P2[sh], Q1[sh], A1[sh], DF(wk.hi, wk.lo), dfs);
-      fo[ip * N] = step_out<L, P, ip, SC>(o.p, p);
-      fo[im * N] = step_out<L, P, im, SC>(o.m, p);
-      return;
-    }
     const R t = edot<L, ip>(cu);
     const R t2 = t * t;
     R ev_in = fma(t2, L::NEQ >= 4 ? fma(t2, P4, P2[sh]) : P2[sh], P0[sh]);
@@ -418,15 +381,97 @@ __device__ __forceinline__ void collide_store(typename Codec<P>::R (&d)[L::Q],
     if constexpr (FO == 3) od_in += stress_pair<L, ip, R>(st);
     const R ev = fma(d[ip] + d[im], hom1, SC ? ev_in : mul_w<L, ip, R, EX>(ev_in));
     const R od = fma(d[ip] - d[im], hom1, SC ? od_in : mul_w<L, ip, R, EX>(od_in));
-    R dp = ev + od, dm = ev - od;
-    if constexpr (P == P_FP64) {
-      if (probe) {
-        dp = probe_round<ip>(dp, p);
-        dm = probe_round<im>(dm, p);
-      }
-    }
-    fo[ip * N] = step_out<L, P, ip, SC>(dp, p);
-    fo[im * N] = step_out<L, P, im, SC>(dm, p);
+    fo[ip * N] = step_out<L, P, ip, SC>(ev + od, p);
+    fo[im * N] = step_out<L, P, im, SC>(ev - od, p);
+  });
+}
+
+// Pair sums s and differences a of the deviations, from the stored values f of
+// an FP64 pull: a = f+ - f- and s = a + 2 (f- - w), three operations a pair
+// where decoding both members takes four.  f+ - f- and f- - w are exact while
+// the members are within a factor of two of each other and of w, so s and a are
+// what the decoded deviations give.
+template <class L, class R>
+__device__ __forceinline__ void pair_split(const R (&f)[L::Q], R& d0, R (&s)[(L::Q - 1) / 2], R (&a)[(L::Q - 1) / 2]) {
+  d0 = f[0] - R(L::W(0));
+  static_for<0, (L::Q - 1) / 2>([&](auto K) {
+    constexpr int k = K, ip = 2 * k + 1;
+    a[k] = f[ip] - f[ip + 1];
+    s[k] = kmac<2>(f[ip + 1] - R(L::W(ip)), a[k]);
+  });
+}
+// The same from deviations (rows at a wall, sites next to solids).
+template <class L, class R>
+__device__ __forceinline__ void pair_split_dev(const R (&d)[L::Q], R& d0, R (&s)[(L::Q - 1) / 2], R (&a)[(L::Q - 1) / 2]) {
+  d0 = d[0];
+  static_for<0, (L::Q - 1) / 2>([&](auto K) {
+    constexpr int k = K, ip = 2 * k + 1;
+    a[k] = d[ip] - d[ip + 1];
+    s[k] = d[ip] + d[ip + 1];
+  });
+}
+
+// Collision of one site of an FP64 grid (IEEE double or float-float) from its
+// pair sums and differences, and store of f*(x): see lbm_poly.cuh.
+template <class L, int P, int FO>
+__device__ __forceinline__ void poly_store(typename Codec<P>::R d0, const typename Codec<P>::R (&s)[(L::Q - 1) / 2],
+                                           const typename Codec<P>::R (&a)[(L::Q - 1) / 2],
+                                           const typename Codec<P>::R (&g)[3], int site,
+                                           typename Codec<P>::T* __restrict__ fout, const StepParams& p) {
+  using C = Codec<P>;
+  using R = typename C::R;
+  constexpr int D = L::D;
+  const size_t N = (size_t)p.N;
+  const RawMoments<L, R> r = pair_moments<L, R>(d0, s, a);
+  // mid-point state (R1): rho, u = u~ + g/2, theta
+  SiteState<R> m;
+  m.drho = r.drho;
+  m.rho = R(1) + r.drho;
+  const R irho = R(1) / m.rho;
+  R u[3] = {R(0), R(0), R(0)};
+  R ut2 = R(0), g2 = R(0), gu = R(0);
+  m.u2 = R(0);
+  for (int c = 0; c < D; ++c) {
+    const R ut = mul_c<L, R>(r.j[c] * irho);
+    u[c] = hmac(g[c], ut);
+    ut2 = c == 0 ? ut * ut : fma(ut, ut, ut2);
+    g2 = c == 0 ? g[c] * g[c] : fma(g[c], g[c], g2);
+    m.u2 = c == 0 ? u[c] * u[c] : fma(u[c], u[c], m.u2);
+    gu = c == 0 ? g[c] * u[c] : fma(g[c], u[c], gu);
+  }
+  m.Th = fma(fma(mul_c2<L, R>(r.k2) - kscale<D>(r.drho), irho, -ut2), R(1.0 / D), g2 * R(0.25 / D));
+  m.om = site_omega<R>(p, m.rho, R(1) + m.Th);
+  m.rom = m.rho * m.om;
+  const R om1 = R(1) - m.om, hom1 = half_of(om1);
+  const R rk = m.rho - half_of(m.rom);
+  m.rkgu = FO >= 1 ? rk * gu : R(0);
+  m.T = mul_c2<L, R>(m.Th);
+  const R crk = mul_c<L, R>(rk);
+  for (int c = 0; c < 3; ++c) {
+    m.U[c] = c < D ? mul_c<L, R>(u[c]) : R(0);
+    m.S[c] = c < D ? crk * g[c] : R(0);
+  }
+  typename std::conditional<D == 2, PolyCoef2<R>, PolyCoef3<R>>::type k;
+  poly_coef<(FO == 3 ? 2 : FO)>(m, k);
+  if constexpr (FO == 3) {
+    R S[6];
+    stress_tensor_pairs<L, R>(s, r.drho, m.rho, m.Th, u, g, S);
+    const R kf = R(1) - half_of(m.om);
+    poly_add_stress(stress_terms<L, R>(S, g, half_of(kf * kf)), k);
+  }
+  typename C::T* __restrict__ fo = fout + site;
+  // FP64 storage probe: the stored deviation rounded as a float codec stores it
+  const bool probe = P == P_FP64 && p.storage_probe != 0;
+  auto put = [&](auto I, R d) {
+    constexpr int i = I;
+    if constexpr (P == P_FP64)
+      if (probe) d = probe_round<i>(d, p);
+    fo[i * N] = C::template encode<L, i>(d, p);
+  };
+  put(ic<0>{}, fma(d0, om1, cmul(L::W(0), const_term(k))));
+  poly_pairs<L, R>(k, hom1, s, a, [&](auto K, R ev, R od) {
+    put(ic<2 * int(K) + 1>{}, ev + od);
+    put(ic<2 * int(K) + 2>{}, ev - od);
   });
 }
 
@@ -444,9 +489,8 @@ __device__ __forceinline__ void collide_store(typename Codec<P>::R (&d)[L::Q],
 #ifndef LBM_FLOAT_D3Q39_BLOCKS
 #define LBM_FLOAT_D3Q39_BLOCKS 3
 #endif
-// LBM_DF_BLOCKS: the same for the float-float FP64 step; 2 (128 registers,
-// ~240 B of spill) measured 1.45x faster than 1 (255 registers) on GB300:
-// the wider kernel hides the instruction-fetch stalls of its long code.
+// LBM_DF_BLOCKS: the same for the float-float FP64 step (2: 128 registers, no
+// spill on D2Q37, ~250 B on D3Q39).
 #ifndef LBM_DF_BLOCKS
 #define LBM_DF_BLOCKS 2
 #endif
@@ -496,12 +540,18 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
     asm volatile("griddepcontrol.wait;" ::: "memory");
     R d[L::Q];
     pull_solid<L, P, R>(fin, p, x, y, z, site, d);
-    collide_store<L, P, FO>(d, g, site, fout, p);
+    if constexpr (P == P_FP64) {
+      R d0, s[(L::Q - 1) / 2], a[(L::Q - 1) / 2];
+      pair_split_dev<L, R>(d, d0, s, a);
+      poly_store<L, P, FO>(d0, s, a, g, site, fout, p);
+    } else {
+      collide_store<L, P, FO>(d, g, site, fout, p);
+    }
     return;
   }
   const int a = L::D == 2 ? y : z;
   const int nA = L::D == 2 ? p.ny : p.nz;
-  const bool near = p.wall != W_NONE && (a < 3 || a >= nA - 3);
+  const bool near = near_wall(p, a, nA);
   const int wx0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31);
   const bool interior = !near && wx0 >= 3 && wx0 + 31 <= p.nx - 4;
   // Programmatic dependent launch: let the next step's blocks be scheduled
@@ -511,11 +561,26 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
   R g[3];
   site_force_r<L::D, R>(p, x, y, z, site, g);
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  constexpr bool SC = scaled_step<P, FO>();
-  R d[L::Q];
-  if (interior) pull_interior<L, P, R, LD_HINT, SC>(fin + site, p, y, z, d);
-  else pull<L, P, R, LD_HINT, SC>(fin, p, x, y, z, d);
-  collide_store<L, P, FO, SC>(d, g, site, fout, p);
+  if constexpr (std::is_same<R, float>::value) {
+    constexpr bool SC = scaled_step<P, FO>();
+    R d[L::Q];
+    if (interior) pull_interior<L, P, R, LD_HINT, SC ? IN_SCALED : IN_DEV>(fin + site, p, y, z, d);
+    else pull<L, P, R, LD_HINT, SC>(fin, p, x, y, z, d);
+    collide_store<L, P, FO, SC>(d, g, site, fout, p);
+  } else {
+    R d0, s[(L::Q - 1) / 2], am[(L::Q - 1) / 2];
+    if (!near) {
+      R f[L::Q];
+      if (interior) pull_interior<L, P, R, LD_HINT, IN_STORED>(fin + site, p, y, z, f);
+      else pull_wrap<L, P, R, LD_HINT, IN_STORED>(fin, p, x, y, z, f);
+      pair_split<L, R>(f, d0, s, am);
+    } else {
+      R d[L::Q];
+      pull<L, P, R>(fin, p, x, y, z, d);
+      pair_split_dev<L, R>(d, d0, s, am);
+    }
+    poly_store<L, P, FO>(d0, s, am, g, site, fout, p);
+  }
 }
 
 // ------------------------------------------------------------ init

@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(WAVE_BX, wave_min_blocks<L, P>())
       site_force_r<D, R>(p, x, y, z, site, g);
       constexpr bool SC = scaled_step<P, FO>();
       R d[L::Q];
-      if (interior) pull_interior<L, P, R, LD_CG, SC>(fin + site, p, y, z, d);
+      if (interior) pull_interior<L, P, R, LD_CG, SC ? IN_SCALED : IN_DEV>(fin + site, p, y, z, d);
       else pull<L, P, R, LD_CG, SC>(fin, p, x, y, z, d);
       collide_store<L, P, FO, SC>(d, g, site, fout, p);
     }
