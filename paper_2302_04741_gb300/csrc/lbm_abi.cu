@@ -576,13 +576,14 @@ int create_impl(lbm_lattice lat, int nx, int ny, int nz, double tau, const lbm_g
   {
     int nsm = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device);
+    c->nsm = nsm;
     const long long tiles = (long long)((nx + 127) / 128) * (D == 2 ? na : (long long)ny * na);
     c->nblk_cons = (int)std::min<long long>(tiles, (long long)LBM_CONSERVED_BLOCKS * (nsm > 0 ? nsm : 1));
   }
   const size_t pb = sizeof(double) * lbm::CONS_SLOT * c->nblk_cons;
   if (cudaMalloc(&c->part, pb) != cudaSuccess || cudaMalloc(&c->bad, sizeof(unsigned) * c->nblk_cons) != cudaSuccess ||
       cudaMalloc(&c->dres, sizeof(double) * (2 * lbm::NCONS + 2)) != cudaSuccess ||
-      cudaMalloc(&c->dmax, sizeof(unsigned)) != cudaSuccess ||
+      cudaMalloc(&c->dmax, sizeof(unsigned) * lbm::MAX_SHELLS) != cudaSuccess ||
       cudaMalloc(&c->ticket, sizeof(unsigned)) != cudaSuccess ||
       cudaMemset(c->ticket, 0, sizeof(unsigned)) != cudaSuccess ||
       cudaMallocHost(&c->hres, sizeof(double) * (2 * lbm::NCONS + 2)) != cudaSuccess) {
@@ -590,7 +591,8 @@ int create_impl(lbm_lattice lat, int nx, int ny, int nz, double tau, const lbm_g
     fail(c, LBM_ENOMEM, "cannot allocate reduction scratch");
     return bail(LBM_ENOMEM);
   }
-  c->bytes += pb + sizeof(unsigned) * c->nblk_cons + sizeof(double) * (2 * lbm::NCONS + 2) + 2 * sizeof(unsigned);
+  c->bytes += pb + sizeof(unsigned) * c->nblk_cons + sizeof(double) * (2 * lbm::NCONS + 2) +
+              (1 + lbm::MAX_SHELLS) * sizeof(unsigned);
   if (cudaMalloc(&c->derr, sizeof(int)) != cudaSuccess || cudaMemset(c->derr, 0, sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
     fail(c, LBM_ENOMEM, "cannot allocate the error flag");
@@ -752,13 +754,17 @@ int lbm_init(lbm_ctx* c, const double* rho, const double* u, const double* T) {
   }
   c->cur = 0;
   if (c->opt.precision == LBM_FP16_SCALED || c->opt.storage_probe == LBM_FP16_SCALED) {
-    LBM_CUDA(c, cudaMemsetAsync(c->dmax, 0, sizeof(unsigned), c->stream));
-    LBM_CUDA(c, c->ops->init(c->opt.precision, 0, drho, du, dT, c->f[0], c->dmax, c->opt.force_order, c->p, c->stream));
-    unsigned bits = 0;
-    LBM_CUDA(c, cudaMemcpyAsync(&bits, c->dmax, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+    unsigned bits[lbm::MAX_SHELLS] = {};
+    LBM_CUDA(c, cudaMemsetAsync(c->dmax, 0, sizeof bits, c->stream));
+    LBM_CUDA(c, c->ops->init_scale(drho, du, dT, c->dmax, c->opt.force_order, c->p, c->nsm, c->stream));
+    LBM_CUDA(c, cudaMemcpyAsync(bits, c->dmax, sizeof bits, cudaMemcpyDeviceToHost, c->stream));
     LBM_CUDA(c, cudaStreamSynchronize(c->stream));
-    float mx;
-    std::memcpy(&mx, &bits, sizeof mx);
+    float mx = 0.f;  // max |d_i / w_i|
+    for (int k = 0; k < c->ops->nshell; ++k) {
+      float d;
+      std::memcpy(&d, &bits[k], sizeof d);
+      mx = std::max(mx, (float)((double)d / c->ops->shell_w[k]));
+    }
     if (!std::isfinite(mx)) return fail(c, LBM_EINVAL, "initial state is not finite");
     // scale s = 2^k with max |d/w| * s in [2^12, 2^13): headroom of 8x below the
     // half-precision maximum for the state to grow into
@@ -772,7 +778,7 @@ int lbm_init(lbm_ctx* c, const double* rho, const double* u, const double* T) {
     c->p.h_inv_scale = std::ldexp(1.0f, -k);
     fp16_factors(c);
   }
-  LBM_CUDA(c, c->ops->init(c->opt.precision, 1, drho, du, dT, c->f[0], nullptr, c->opt.force_order, c->p, c->stream));
+  LBM_CUDA(c, c->ops->init(c->opt.precision, drho, du, dT, c->f[0], c->opt.force_order, c->p, c->stream));
   // host arrays (staged or read in place) may be freed after return
   if (!is_device_ptr(rho) || !is_device_ptr(u) || !is_device_ptr(T))
     LBM_CUDA(c, cudaStreamSynchronize(c->stream));

@@ -47,10 +47,11 @@ struct lbm_ctx {
   unsigned* bad = nullptr;     // bad-site counts per block
   double* dres = nullptr;      // final reduction result (when hres is not mapped)
   unsigned* ticket = nullptr;  // last-block ticket of the conservation pass
-  unsigned* dmax = nullptr;    // FP16 init: max |d/w| bits
+  unsigned* dmax = nullptr;    // FP16 init: max |d| bits per shell
   double* hres = nullptr;      // pinned host copy of the result
   double* tmp = nullptr;       // (2 + 2D) * N doubles, lazily allocated
   int nblk_cons = 0;
+  int nsm = 0;                 // multiprocessors of the device
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   lbm::StepParams p{};

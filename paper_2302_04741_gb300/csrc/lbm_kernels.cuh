@@ -72,10 +72,10 @@ __device__ __forceinline__ typename Codec<P>::R pulled_value(typename Codec<P>::
   else return step_in<L, P, I, IN == IN_SCALED>(v, p);
 }
 
-// Pull of all Q populations of site (x, y, z) of a row that no wall rule
+// Pull of the stored values of site (x, y, z) of a row that no wall rule
 // touches, with the periodic wrap of every axis.
-template <class L, int P, class RR, int LD = LD_HINT, int IN = IN_DEV>
-__device__ __forceinline__ void pull_wrap(const typename Codec<P>::T* __restrict__ fin,
+template <class L, int P, class RR, int LD = LD_HINT>
+__device__ __forceinline__ void pull_stored(const typename Codec<P>::T* __restrict__ fin,
                                           const StepParams& p, int x, int y, int z, RR (&d)[L::Q]) {
   using C = Codec<P>;
   constexpr int D = L::D, Q = L::Q;
@@ -92,7 +92,7 @@ __device__ __forceinline__ void pull_wrap(const typename Codec<P>::T* __restrict
     constexpr int i = I;
     constexpr int ex = L::E(i, 0), ey = L::E(i, 1), ez = L::E(i, 2);
     const int off = zs[ez + 3] + ys[ey + 3] + xs[ex + 3];
-    d[i] = RR(pulled_value<L, P, i, IN>(ldpop<C, LD>(fin + i * N + off, p), p));
+    d[i] = pulled_value<L, P, i, IN_STORED>(ldpop<C, LD>(fin + i * N + off, p), p);
   });
 }
 
@@ -113,16 +113,21 @@ __device__ __forceinline__ void pull(const typename Codec<P>::T* __restrict__ fi
   const size_t N = (size_t)p.N;
   const int a = D == 2 ? y : z;          // coordinate along the wall axis
   const int nA = D == 2 ? ny : nz;
-  if (!near_wall(p, a, nA)) {
-    pull_wrap<L, P, RR, LD, SC ? IN_SCALED : IN_DEV>(fin, p, x, y, z, d);
-    return;
-  }
   int xs[7], ys[7], zs[7];
 #pragma unroll
   for (int k = 0; k < 7; ++k) {
     xs[k] = wrap3(x - (k - 3), nx);
     ys[k] = wrap3(y - (k - 3), ny) * nx;
     zs[k] = D == 3 ? wrap3(z - (k - 3), nz) * nx * ny : 0;
+  }
+  if (!near_wall(p, a, nA)) {
+    static_for<0, Q>([&](auto I) {
+      constexpr int i = I;
+      constexpr int ex = L::E(i, 0), ey = L::E(i, 1), ez = L::E(i, 2);
+      const int off = zs[ez + 3] + ys[ey + 3] + xs[ex + 3];
+      d[i] = RR(step_in<L, P, i, SC>(ldpop<C, LD>(fin + i * N + off, p), p));
+    });
+    return;
   }
   // ---- a row next to a wall: slots whose source lies beyond the wall
   const int side = a < 3 ? 0 : 1;
@@ -469,9 +474,11 @@ __device__ __forceinline__ void poly_store(typename Codec<P>::R d0, const typena
     fo[i * N] = C::template encode<L, i>(d, p);
   };
   put(ic<0>{}, fma(d0, om1, cmul(L::W(0), const_term(k))));
-  poly_pairs<L, R>(k, hom1, s, a, [&](auto K, R ev, R od) {
-    put(ic<2 * int(K) + 1>{}, ev + od);
-    put(ic<2 * int(K) + 2>{}, ev - od);
+  poly_pairs<L, R>(k, [&](auto K, R wev, R wod) {
+    constexpr int kp = K;
+    const R ev = fma(hom1, s[kp], wev), od = fma(hom1, a[kp], wod);
+    put(ic<2 * kp + 1>{}, ev + od);
+    put(ic<2 * kp + 2>{}, ev - od);
   });
 }
 
@@ -572,7 +579,7 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
     if (!near) {
       R f[L::Q];
       if (interior) pull_interior<L, P, R, LD_HINT, IN_STORED>(fin + site, p, y, z, f);
-      else pull_wrap<L, P, R, LD_HINT, IN_STORED>(fin, p, x, y, z, f);
+      else pull_stored<L, P, R>(fin, p, x, y, z, f);
       pair_split<L, R>(f, d0, s, am);
     } else {
       R d[L::Q];
@@ -587,7 +594,7 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
 // f~_i = f0_i(rho, u, T) - F_i(rho, u, T)/2 as deviations
 // d_i = w_i [drho + rho (p_i - F'_i/2)], placed at the slot the next pull of
 // (x, i) reads: x - e_i (periodic), or the mirrored slot of the opposite
-// direction beyond a wall.  MODE 0 only records max |d_i / w_i| (FP16 scale).
+// direction beyond a wall.
 template <class L, int FO, class R>
 __device__ __forceinline__ void init_site(const MidState<L, R>& m, R (&d)[L::Q]) {
   constexpr int NP = (L::Q - 1) / 2;
@@ -607,13 +614,108 @@ __device__ __forceinline__ void init_site(const MidState<L, R>& m, R (&d)[L::Q])
   });
 }
 
-template <class L, int P, int MODE>
-__global__ void __launch_bounds__(128) k_init(const double* __restrict__ rho,
-                                              const double* __restrict__ u,
-                                              const double* __restrict__ T,
-                                              typename Codec<P>::T* __restrict__ fout,
-                                              unsigned int* __restrict__ maxbits, int force_order,
-                                              const StepParams p) {
+// The same in double, by parity classes (lbm_poly.cuh): the polynomial of the
+// step with om = 1 and the force's factor 1 - om/2 replaced by -1/2.
+template <class L, int FO>
+__device__ __forceinline__ void init_site_poly(double drho, const double (&u)[3], double Th, const double (&g)[3],
+                                               double (&d)[L::Q]) {
+  constexpr int D = L::D;
+  SiteState<double> m;
+  m.drho = drho;
+  m.rho = 1.0 + drho;
+  m.om = 1.0;
+  m.Th = Th;
+  m.T = L::c2 * Th;
+  m.rom = m.rho;
+  m.u2 = 0.0;
+  const double rk = -0.5 * m.rho;
+  double gu = 0.0;
+  for (int c = 0; c < 3; ++c) {
+    m.U[c] = c < D ? L::c * u[c] : 0.0;
+    m.S[c] = c < D ? L::c * rk * g[c] : 0.0;
+    if (c < D) {
+      m.u2 = fma(u[c], u[c], m.u2);
+      gu = fma(g[c], u[c], gu);
+    }
+  }
+  m.rkgu = rk * gu;
+  typename std::conditional<D == 2, PolyCoef2<double>, PolyCoef3<double>>::type k;
+  poly_coef<FO>(m, k);
+  d[0] = L::W(0) * const_term(k);
+  poly_pairs<L, double>(k, [&](auto K, double ev, double od) {
+    d[2 * int(K) + 1] = ev + od;
+    d[2 * int(K) + 2] = ev - od;
+  });
+}
+
+// Deviations of site (x, y, z) from the given fields.
+template <class L, class R>
+__device__ __forceinline__ void init_deviations(const double* __restrict__ rho, const double* __restrict__ u,
+                                                const double* __restrict__ T, int force_order, const StepParams& p,
+                                                int x, int y, int z, int site, R (&d)[L::Q]) {
+  constexpr int D = L::D;
+  const size_t N = (size_t)p.N;
+  double gd[3];
+  site_force<D>(p, x, y, z, site, gd);
+  if constexpr (std::is_same<R, double>::value) {
+    const double uu[3] = {u[site], u[N + site], D == 3 ? u[2 * N + site] : 0.0};
+    const double drho = rho[site] - 1.0, Th = T[site] - 1.0;
+    if (force_order == 0) init_site_poly<L, 0>(drho, uu, Th, gd, d);
+    else if (force_order == 1) init_site_poly<L, 1>(drho, uu, Th, gd, d);
+    else init_site_poly<L, 2>(drho, uu, Th, gd, d);
+  } else {
+    const R g[3] = {R(gd[0]), R(gd[1]), R(gd[2])};
+    const R uu[3] = {R(u[site]), R(u[N + site]), D == 3 ? R(u[2 * N + site]) : R(0)};
+    MidState<L, R> m;
+    given_state<L, R>(R(rho[site] - 1.0), uu, R(T[site] - 1.0), g, m);
+    if (force_order == 0) init_site<L, 0, R>(m, d);
+    else if (force_order == 1) init_site<L, 1, R>(m, d);
+    else init_site<L, 2, R>(m, d);
+  }
+}
+
+// Largest |d_i| of each shell of directions over the sites an FP16 grid
+// initialises (as bits; maxbits: L::NSHELL zeroed words): the host divides it
+// by the shell's weight for the scale.  (Rounding is monotonic, so this is the
+// largest rounded |d_i / w_i|, without a double division per population; and
+// one atomic per block and shell instead of one per site.  512 x 512 x 256
+// sites: 47.8 ms before.)
+template <class L>
+__global__ void __launch_bounds__(256) k_init_scale(const double* __restrict__ rho, const double* __restrict__ u,
+                                                    const double* __restrict__ T, unsigned int* __restrict__ maxbits,
+                                                    int force_order, const StepParams p) {
+  constexpr int D = L::D;
+  const int layer = D == 2 ? p.nx : p.nx * p.ny;
+  const int end = (p.a0 + p.na) * layer;
+  float mx[L::NSHELL];
+  for (int k = 0; k < L::NSHELL; ++k) mx[k] = 0.f;
+  // (long long: site + stride may pass 2^31)
+  for (long long s = (long long)p.a0 * layer + blockIdx.x * 256 + threadIdx.x; s < end; s += (long long)gridDim.x * 256) {
+    const int site = (int)s;
+    if (p.solid && p.solid[site]) continue;
+    const int x = site % p.nx, row = site / p.nx;
+    float d[L::Q];
+    init_deviations<L, float>(rho, u, T, force_order, p, x, row % p.ny, row / p.ny, site, d);
+    static_for<0, L::Q>([&](auto I) {
+      constexpr int i = I;
+      mx[L::SH(i)] = fmaxf(mx[L::SH(i)], fabsf(d[i]));
+    });
+  }
+  __shared__ unsigned sh[L::NSHELL];
+  if (threadIdx.x < L::NSHELL) sh[threadIdx.x] = 0u;
+  __syncthreads();
+  for (int k = 0; k < L::NSHELL; ++k) {
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(mx[k]));
+    if ((threadIdx.x & 31) == 0) atomicMax(sh + k, m);
+  }
+  __syncthreads();
+  if (threadIdx.x < L::NSHELL) atomicMax(maxbits + threadIdx.x, sh[threadIdx.x]);
+}
+
+template <class L, int P>
+__global__ void __launch_bounds__(128) k_init(const double* __restrict__ rho, const double* __restrict__ u,
+                                              const double* __restrict__ T, typename Codec<P>::T* __restrict__ fout,
+                                              int force_order, const StepParams p) {
   using C = Codec<P>;
   using R = typename C::R;
   constexpr int Q = L::Q, D = L::D;
@@ -625,29 +727,10 @@ __global__ void __launch_bounds__(128) k_init(const double* __restrict__ rho,
   const int site = (z * ny + y) * nx + x;
   const size_t N = (size_t)p.N;
   if (p.solid && p.solid[site]) return;
-  double gd[3];
-  site_force<D>(p, x, y, z, site, gd);
-  const R g[3] = {R(gd[0]), R(gd[1]), R(gd[2])};
-  const R uu[3] = {R(u[site]), R(u[N + site]), D == 3 ? R(u[2 * N + site]) : R(0)};
-  MidState<L, R> m;
-  given_state<L, R>(R(rho[site] - 1.0), uu, R(T[site] - 1.0), g, m);
   R d[Q];
-  if (force_order == 0) init_site<L, 0, R>(m, d);
-  else if (force_order == 1) init_site<L, 1, R>(m, d);
-  else init_site<L, 2, R>(m, d);
-  if (MODE == 0) {
-    float mx = 0.f;
-    static_for<0, Q>([&](auto I) {
-      constexpr int i = I;
-      mx = fmaxf(mx, (float)fabs(double(d[i]) / L::W(i)));
-    });
-    atomicMax(maxbits, __float_as_uint(mx));
-    return;
-  }
+  init_deviations<L, R>(rho, u, T, force_order, p, x, y, z, site, d);
   const int a = D == 2 ? y : z;
   const int nA = D == 2 ? ny : nz;
-  const int lineA = D == 2 ? nx : nx * ny;
-  const int colbase = D == 2 ? x : (y * nx + x);
   if constexpr (P == P_FP64) {  // storage probe: the initial state as a float codec stores it
     if (p.storage_probe)
       static_for<0, Q>([&](auto I) {
@@ -655,6 +738,22 @@ __global__ void __launch_bounds__(128) k_init(const double* __restrict__ rho,
         d[i] = probe_round<i>(d[i], p);
       });
   }
+  if (!near_wall(p, a, nA) && !p.solid) {  // block-uniform: the slots a plain pull reads
+    int xs[7], ys[7], zs[7];
+#pragma unroll
+    for (int k = 0; k < 7; ++k) {
+      xs[k] = wrap3(x - (k - 3), nx);
+      ys[k] = wrap3(y - (k - 3), ny) * nx;
+      zs[k] = D == 3 ? wrap3(z - (k - 3), nz) * nx * ny : 0;
+    }
+    static_for<0, Q>([&](auto I) {
+      constexpr int i = I;
+      fout[i * N + (zs[L::E(i, 2) + 3] + ys[L::E(i, 1) + 3] + xs[L::E(i, 0) + 3])] = C::template encode<L, i>(d[i], p);
+    });
+    return;
+  }
+  const int lineA = D == 2 ? nx : nx * ny;
+  const int colbase = D == 2 ? x : (y * nx + x);
   static_for<0, Q>([&](auto I) {
     constexpr int i = I;
     constexpr int ex = L::E(i, 0), ey = L::E(i, 1), ez = L::E(i, 2);

@@ -11,13 +11,21 @@
 
 namespace lbm {
 
+constexpr int MAX_SHELLS = 8;  // of a lattice's directions
+
 // Function table of one lattice, filled by lattice_ops<L>().
 struct LatticeOps {
   int Q, D;
   cudaError_t (*step)(int P, int FO, const void* fin, void* fout, const StepParams& p, int bx,
                       bool overlap, cudaStream_t s);  // p.solid set: FP64 / FP32 only
-  cudaError_t (*init)(int P, int mode, const double* rho, const double* u, const double* T,
-                      void* fout, unsigned* maxbits, int FO, const StepParams& p, cudaStream_t s);
+  cudaError_t (*init)(int P, const double* rho, const double* u, const double* T, void* fout, int FO,
+                      const StepParams& p, cudaStream_t s);
+  // largest |d_i| per shell (bits) over the initial state, for the FP16 scale;
+  // maxbits: MAX_SHELLS zeroed words, w[shell] the weights
+  cudaError_t (*init_scale)(const double* rho, const double* u, const double* T, unsigned* maxbits, int FO,
+                            const StepParams& p, int nsm, cudaStream_t s);
+  int nshell;
+  const double* shell_w;
   cudaError_t (*moments)(int P, const void* fin, double* rho, double* u, double* T, double* q,
                          int FO, const StepParams& p, cudaStream_t s);
   // ticket != nullptr: the last block also reduces into out (see k_conserved)
@@ -148,19 +156,21 @@ struct Ops {
     return e != cudaSuccess ? e : cudaGetLastError();
   }
 
-  static cudaError_t init(int P, int mode, const double* rho, const double* u, const double* T_,
-                          void* fout, unsigned* maxbits, int FO, const StepParams& p,
-                          cudaStream_t s) {
+  static cudaError_t init(int P, const double* rho, const double* u, const double* T_, void* fout, int FO,
+                          const StepParams& p, cudaStream_t s) {
     const dim3 g = row_grid<L::D>(p, 128), b(128);
-    if (mode == 0) {
-      k_init<L, P_FP16S, 0><<<g, b, 0, s>>>(rho, u, T_, (T<P_FP16S>*)fout, maxbits, FO, p);
-    } else if (P == P_FP64) {
-      k_init<L, P_FP64, 1><<<g, b, 0, s>>>(rho, u, T_, (T<P_FP64>*)fout, maxbits, FO, p);
-    } else if (P == P_FP32S) {
-      k_init<L, P_FP32S, 1><<<g, b, 0, s>>>(rho, u, T_, (T<P_FP32S>*)fout, maxbits, FO, p);
-    } else {
-      k_init<L, P_FP16S, 1><<<g, b, 0, s>>>(rho, u, T_, (T<P_FP16S>*)fout, maxbits, FO, p);
-    }
+    if (P == P_FP64) k_init<L, P_FP64><<<g, b, 0, s>>>(rho, u, T_, (T<P_FP64>*)fout, FO, p);
+    else if (P == P_FP32S) k_init<L, P_FP32S><<<g, b, 0, s>>>(rho, u, T_, (T<P_FP32S>*)fout, FO, p);
+    else k_init<L, P_FP16S><<<g, b, 0, s>>>(rho, u, T_, (T<P_FP16S>*)fout, FO, p);
+    return cudaGetLastError();
+  }
+
+  static cudaError_t init_scale(const double* rho, const double* u, const double* T_, unsigned* maxbits, int FO,
+                                const StepParams& p, int nsm, cudaStream_t s) {
+    const long long sites = (long long)p.na * (L::D == 2 ? p.nx : p.nx * p.ny);
+    const long long most = 4LL * (nsm > 0 ? nsm : 1);
+    const unsigned blocks = (unsigned)((sites + 255) / 256 < most ? (sites + 255) / 256 : most);
+    k_init_scale<L><<<blocks, 256, 0, s>>>(rho, u, T_, maxbits, FO, p);
     return cudaGetLastError();
   }
 
@@ -363,7 +373,7 @@ struct Ops {
   }
 
   static LatticeOps table() {
-    return LatticeOps{L::Q, L::D, &step, &init, &moments, &conserved, &conserved_final, &pulled, &state,
+    return LatticeOps{L::Q, L::D, &step, &init, &init_scale, L::NSHELL, L::shell_w, &moments, &conserved, &conserved_final, &pulled, &state,
                       &tma_smem, &tma_prepare, &step_tma, &async_occupancy, &step_async,
                       &batch_occupancy, &batch_step, &batch_staged_occupancy, &batch_step_staged,
                       &wave_occupancy, &step_wave};

@@ -276,14 +276,11 @@ __device__ __forceinline__ void poly_add_stress(const StressTerms<R>& st, PolyCo
   k.o111 = kmac<2>(c, k.o111);
 }
 
-// Even and odd part of w G at every pair, handed to out(pair, ev, od) with
-// ev, od the pair's values of hom1 s + w G_even and hom1 a + w G_odd.
+// Even and odd part of w G at every pair, handed to out(pair, w G_even, w G_odd).
 template <class L, class R, class OUT>
-__device__ __forceinline__ void poly_pairs(const PolyCoef2<R>& k, R hom1, const R (&s)[(L::Q - 1) / 2],
-                                           const R (&a)[(L::Q - 1) / 2], OUT&& out) {
+__device__ __forceinline__ void poly_pairs(const PolyCoef2<R>& k, OUT&& out) {
   auto pair = [&](auto X, auto Y, R wev, R wod) {
-    constexpr int kp = pair_of<L>(X, Y, 0);
-    out(ic<kp>{}, fma(hom1, s[kp], wev), fma(hom1, a[kp], wod));
+    out(ic<pair_of<L>(X, Y, 0)>{}, wev, wod);
   };
   static_for<0, 4>([&](auto A) {
     constexpr int aa = A * A;
@@ -317,11 +314,9 @@ __device__ __forceinline__ void poly_pairs(const PolyCoef2<R>& k, R hom1, const 
 }
 
 template <class L, class R, class OUT>
-__device__ __forceinline__ void poly_pairs(const PolyCoef3<R>& k, R hom1, const R (&s)[(L::Q - 1) / 2],
-                                           const R (&a)[(L::Q - 1) / 2], OUT&& out) {
+__device__ __forceinline__ void poly_pairs(const PolyCoef3<R>& k, OUT&& out) {
   auto pair = [&](auto X, auto Y, auto Z, R wev, R wod) {
-    constexpr int kp = pair_of<L>(X, Y, Z);
-    out(ic<kp>{}, fma(hom1, s[kp], wev), fma(hom1, a[kp], wod));
+    out(ic<pair_of<L>(X, Y, Z)>{}, wev, wod);
   };
   constexpr ic<0> _0{};
   constexpr ic<1> _1{};
