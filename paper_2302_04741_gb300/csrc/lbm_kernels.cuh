@@ -795,120 +795,141 @@ __global__ void __launch_bounds__(128) k_init(const double* __restrict__ rho, co
 // which is (D + 2) rho theta g_a at order 2.  sum f~ |c|^2 c comes from the
 // raw moments of the deviations d = f~ - w: m0 = sum d, m1 = sum d e,
 // m2 = sum d e e, m3 = sum d |e|^2 e (c = xi - u, xi = c_lat e).
-template <class L>
+//
+// The sums run over mirror groups first (as pair_moments, lbm_poly.cuh): a
+// group's even and odd parts feed all moments, so a group of four directions
+// takes 4 additions and some 9 more instead of 4 + 8 per pair.
+template <class R>
 struct HeatMoments {
-  double m0, m1[3], m2[6], m3[3];  // m2 as (xx, yy, zz, xy, xz, yz)
+  R m0, m1[3], m2[6], m3[3];  // m2 as (xx, yy, zz, xy, xz, yz)
 };
 
-template <class L>
-__device__ __forceinline__ HeatMoments<L> heat_moments(const double (&d)[L::Q]) {
-  constexpr int NP = (L::Q - 1) / 2;
-  HeatMoments<L> h{};
-  h.m0 = d[0];
-  static_for<0, NP>([&](auto K) {
-    constexpr int ip = 2 * K + 1, im = ip + 1;
-    constexpr int ex = L::E(ip, 0), ey = L::E(ip, 1), ez = L::E(ip, 2);
-    constexpr int e2 = ex * ex + ey * ey + ez * ez;
-    const double s = d[ip] + d[im];
-    const double a = d[ip] - d[im];
-    h.m0 += s;
-    h.m1[0] = mac<ex>(a, h.m1[0]);
-    h.m1[1] = mac<ey>(a, h.m1[1]);
-    h.m2[0] = mac<ex * ex>(s, h.m2[0]);
-    h.m2[1] = mac<ey * ey>(s, h.m2[1]);
-    h.m2[3] = mac<ex * ey>(s, h.m2[3]);
-    h.m3[0] = mac<e2 * ex>(a, h.m3[0]);
-    h.m3[1] = mac<e2 * ey>(a, h.m3[1]);
-    if constexpr (L::D == 3) {
-      h.m1[2] = mac<ez>(a, h.m1[2]);
-      h.m2[2] = mac<ez * ez>(s, h.m2[2]);
-      h.m2[4] = mac<ex * ez>(s, h.m2[4]);
-      h.m2[5] = mac<ey * ez>(s, h.m2[5]);
-      h.m3[2] = mac<e2 * ez>(a, h.m3[2]);
-    }
-  });
-  return h;
-}
-
-// The same raw moments from float deviations without FP64 arithmetic: each
-// moment is a float pair s + c, the pair sums d_+ +- d_- are split exactly
-// (Knuth's two-sum), products by the small integer weights keep their FMA
-// residual, and every rounding error goes into c.  The result equals the
-// FP64 sum to a few units in 2^-48 of the terms' magnitude.
+// An unevaluated sum s + c of two floats as an accumulator: the rounding
+// error of every addition goes into c (Knuth's two-sum), which is not
+// renormalised, so an addition takes 8 instructions; the result equals the
+// FP64 sum to a few units in 2^-48 of the terms' magnitude.  (Explicit
+// round-to-nearest operations: a product fused into a following sum would
+// break the error-free transformations.)
 struct FF {
   float s = 0.f, c = 0.f;
 };
-// (explicit round-to-nearest operations: a product fused into a following
-// sum would break these error-free transformations)
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+__device__ __forceinline__ FF operator+(FF a, FF b) {
+  FF r;
+  float e;
+  df_two_sum(a.s, b.s, r.s, e);
+  r.c = __fadd_rn(__fadd_rn(a.c, b.c), e);
+  return r;
 }
-// acc += K (hi + lo) for a compile-time integer K
+__device__ __forceinline__ FF operator-(FF a, FF b) { return a + FF{-b.s, -b.c}; }
+// acc + K v for a compile-time integer K
 template <int K>
-__device__ __forceinline__ void ff_mac(FF& acc, float hi, float lo) {
-  if constexpr (K != 0) {
-    const float p = __fmul_rn(float(K), hi);
-    const float pe = fmaf(float(K), hi, -p);
-    float t, e;
-    two_sum(acc.s, p, t, e);
-    acc.s = t;
-    acc.c += e + pe + float(K) * lo;
+__device__ __forceinline__ FF kmac(FF v, FF acc) {
+  if constexpr (K == 1) {
+    return acc + v;
+  } else {
+    const float p = __fmul_rn(float(K), v.s);
+    const float pe = (K & (K - 1)) == 0 ? 0.f : fmaf(float(K), v.s, -p);
+    return acc + FF{p, (K & (K - 1)) == 0 ? __fmul_rn(float(K), v.c) : fmaf(float(K), v.c, pe)};
   }
 }
 
-// Symmetric 3x3 (xx, yy, zz, xy, xz, yz) times a vector.
-template <class R>
-__device__ __forceinline__ void sym_mul(const R (&S)[6], const R (&v)[3], R (&o)[3]) {
-  o[0] = S[0] * v[0] + S[3] * v[1] + S[4] * v[2];
-  o[1] = S[3] * v[0] + S[1] * v[1] + S[5] * v[2];
-  o[2] = S[4] * v[0] + S[5] * v[1] + S[2] * v[2];
+// The raw moments from the rest deviation and the pair sums s and differences
+// a, in double or as FF pairs.
+template <class L, class R>
+__device__ __forceinline__ HeatMoments<R> heat_moments(R d0, const R (&s)[(L::Q - 1) / 2], const R (&a)[(L::Q - 1) / 2]) {
+  HeatMoments<R> h{};
+  if constexpr (L::D == 2) {
+    // even part, and the parts odd in x and y, odd in x, odd in y, of the group (+-X, +-Y)
+    auto S = [&](auto X, auto Y) { return at<L, X, Y, 0>(s) + at<L, X, -Y, 0>(s); };
+    auto O = [&](auto X, auto Y) { return at<L, X, Y, 0>(s) - at<L, X, -Y, 0>(s); };
+    auto Ax = [&](auto X, auto Y) { return at<L, X, Y, 0>(a) + at<L, X, -Y, 0>(a); };
+    auto Ay = [&](auto X, auto Y) { return at<L, X, Y, 0>(a) - at<L, X, -Y, 0>(a); };
+    constexpr ic<1> _1{};
+    constexpr ic<2> _2{};
+    constexpr ic<3> _3{};
+    {
+      const R s11 = S(_1, _1), s12 = S(_1, _2), s21 = S(_2, _1), s22 = S(_2, _2), s13 = S(_1, _3), s31 = S(_3, _1);
+      // sums over |e_x| = 1, 2, 3, and over |e_y|
+      const R x1 = (at<L, 1, 0, 0>(s) + s11) + (s12 + s13), x2 = at<L, 2, 0, 0>(s) + (s21 + s22), x3 = at<L, 3, 0, 0>(s) + s31;
+      const R y1 = (at<L, 0, 1, 0>(s) + s11) + (s21 + s31), y2 = at<L, 0, 2, 0>(s) + (s12 + s22), y3 = at<L, 0, 3, 0>(s) + s13;
+      const R x0 = (d0 + at<L, 0, 1, 0>(s)) + (at<L, 0, 2, 0>(s) + at<L, 0, 3, 0>(s));
+      h.m0 = (x0 + x1) + (x2 + x3);
+      h.m2[0] = kmac<9>(x3, kmac<4>(x2, x1));
+      h.m2[1] = kmac<9>(y3, kmac<4>(y2, y1));
+    }
+    h.m2[3] = kmac<4>(O(_2, _2), kmac<3>(O(_1, _3) + O(_3, _1), kmac<2>(O(_1, _2) + O(_2, _1), O(_1, _1))));
+    // sum d e_x and sum d |e|^2 e_x, |e|^2 e_x = e_x^3 + e_x e_y^2
+    auto odd = [&](R p1, R p2, R p3, R p11, R p12, R p13, R p21, R p22, R p31, R& m1, R& m3) {
+      const R x1 = (p1 + p11) + (p12 + p13), x2 = p2 + (p21 + p22), x3 = p3 + p31;
+      m1 = kmac<3>(x3, kmac<2>(x2, x1));
+      const R c1 = kmac<9>(p13, kmac<4>(p12, p11)), c2 = kmac<4>(p22, p21);  // sums of e_y^2
+      m3 = kmac<27>(x3, kmac<8>(x2, x1)) + kmac<3>(p31, kmac<2>(c2, c1));
+    };
+    odd(at<L, 1, 0, 0>(a), at<L, 2, 0, 0>(a), at<L, 3, 0, 0>(a), Ax(_1, _1), Ax(_1, _2), Ax(_1, _3), Ax(_2, _1), Ax(_2, _2),
+        Ax(_3, _1), h.m1[0], h.m3[0]);
+    odd(at<L, 0, 1, 0>(a), at<L, 0, 2, 0>(a), at<L, 0, 3, 0>(a), Ay(_1, _1), Ay(_2, _1), Ay(_3, _1), Ay(_1, _2), Ay(_2, _2),
+        Ay(_1, _3), h.m1[1], h.m3[1]);
+  } else {
+    // (1, 1, 1) and its mirrors: even part and the parts odd in two components
+    const R ep = at<L, 1, 1, 1>(s) + at<L, 1, 1, -1>(s), eq = at<L, 1, -1, 1>(s) + at<L, 1, -1, -1>(s);
+    const R em = at<L, 1, 1, 1>(s) - at<L, 1, 1, -1>(s), en = at<L, 1, -1, 1>(s) - at<L, 1, -1, -1>(s);
+    const R s3 = ep + eq;
+    const R pxy = at<L, 2, 2, 0>(s) + at<L, 2, -2, 0>(s), pxz = at<L, 2, 0, 2>(s) + at<L, 2, 0, -2>(s),
+            pyz = at<L, 0, 2, 2>(s) + at<L, 0, 2, -2>(s);
+    h.m2[3] = kmac<4>(at<L, 2, 2, 0>(s) - at<L, 2, -2, 0>(s), ep - eq);
+    h.m2[4] = kmac<4>(at<L, 2, 0, 2>(s) - at<L, 2, 0, -2>(s), em + en);
+    h.m2[5] = kmac<4>(at<L, 0, 2, 2>(s) - at<L, 0, 2, -2>(s), em - en);
+    const R q2x = at<L, 2, 0, 0>(s), q2y = at<L, 0, 2, 0>(s), q2z = at<L, 0, 0, 2>(s);
+    h.m2[0] = kmac<9>(at<L, 3, 0, 0>(s), kmac<4>(q2x + (pxy + pxz), at<L, 1, 0, 0>(s) + s3));
+    h.m2[1] = kmac<9>(at<L, 0, 3, 0>(s), kmac<4>(q2y + (pxy + pyz), at<L, 0, 1, 0>(s) + s3));
+    h.m2[2] = kmac<9>(at<L, 0, 0, 3>(s), kmac<4>(q2z + (pxz + pyz), at<L, 0, 0, 1>(s) + s3));
+    const R s1 = (at<L, 1, 0, 0>(s) + at<L, 0, 1, 0>(s)) + at<L, 0, 0, 1>(s);
+    const R s9 = (at<L, 3, 0, 0>(s) + at<L, 0, 3, 0>(s)) + at<L, 0, 0, 3>(s);
+    h.m0 = ((d0 + s1) + (s3 + s9)) + (((q2x + q2y) + q2z) + ((pxy + pxz) + pyz));
+    const R u = at<L, 1, 1, 1>(a) + at<L, 1, 1, -1>(a), v = at<L, 1, -1, 1>(a) + at<L, 1, -1, -1>(a);
+    const R x = at<L, 1, 1, 1>(a) - at<L, 1, 1, -1>(a), y = at<L, 1, -1, 1>(a) - at<L, 1, -1, -1>(a);
+    // axes a1, a2, a3; o the octet (|e|^2 = 3), p the planes (|e|^2 = 8, component 2)
+    auto odd = [&](R a1, R a2, R a3, R o, R p, R& m1, R& m3) {
+      m1 = kmac<3>(a3, kmac<2>(a2 + p, a1 + o));
+      m3 = kmac<27>(a3, kmac<16>(p, kmac<8>(a2, kmac<3>(o, a1))));
+    };
+    odd(at<L, 1, 0, 0>(a), at<L, 2, 0, 0>(a), at<L, 3, 0, 0>(a), u + v,
+        (at<L, 2, 2, 0>(a) + at<L, 2, -2, 0>(a)) + (at<L, 2, 0, 2>(a) + at<L, 2, 0, -2>(a)), h.m1[0], h.m3[0]);
+    odd(at<L, 0, 1, 0>(a), at<L, 0, 2, 0>(a), at<L, 0, 3, 0>(a), u - v,
+        (at<L, 2, 2, 0>(a) - at<L, 2, -2, 0>(a)) + (at<L, 0, 2, 2>(a) + at<L, 0, 2, -2>(a)), h.m1[1], h.m3[1]);
+    odd(at<L, 0, 0, 1>(a), at<L, 0, 0, 2>(a), at<L, 0, 0, 3>(a), x + y,
+        (at<L, 2, 0, 2>(a) - at<L, 2, 0, -2>(a)) + (at<L, 0, 2, 2>(a) - at<L, 0, 2, -2>(a)), h.m1[2], h.m3[2]);
+  }
+  return h;
 }
 
-// The same raw moments as float-float values: each compensated pair s + c
+// The float deviations' moments as float-float values: FF sums, each
 // renormalised (an exact two-sum, since c may exceed ulp(s) after a
 // cancellation).
 template <class L>
-__device__ __forceinline__ void heat_moments_df(const float (&d)[L::Q], DF& m0, DF (&m1)[3], DF (&m2)[6],
-                                                DF (&m3)[3]) {
+__device__ __forceinline__ HeatMoments<DF> heat_moments_df(const float (&d)[L::Q]) {
   constexpr int NP = (L::Q - 1) / 2;
-  FF f0, f1[3], f2[6], f3[3];
-  f0.s = d[0];
+  FF s[NP], a[NP];
   static_for<0, NP>([&](auto K) {
-    constexpr int ip = 2 * K + 1, im = ip + 1;
-    constexpr int ex = L::E(ip, 0), ey = L::E(ip, 1), ez = L::E(ip, 2);
-    constexpr int e2 = ex * ex + ey * ey + ez * ez;
-    float sh, sl, ah, al;
-    two_sum(d[ip], d[im], sh, sl);
-    two_sum(d[ip], -d[im], ah, al);
-    ff_mac<1>(f0, sh, sl);
-    ff_mac<ex>(f1[0], ah, al);
-    ff_mac<ey>(f1[1], ah, al);
-    ff_mac<ex * ex>(f2[0], sh, sl);
-    ff_mac<ey * ey>(f2[1], sh, sl);
-    ff_mac<ex * ey>(f2[3], sh, sl);
-    ff_mac<e2 * ex>(f3[0], ah, al);
-    ff_mac<e2 * ey>(f3[1], ah, al);
-    if constexpr (L::D == 3) {
-      ff_mac<ez>(f1[2], ah, al);
-      ff_mac<ez * ez>(f2[2], sh, sl);
-      ff_mac<ex * ez>(f2[4], sh, sl);
-      ff_mac<ey * ez>(f2[5], sh, sl);
-      ff_mac<e2 * ez>(f3[2], ah, al);
-    }
+    constexpr int k = K, ip = 2 * k + 1;
+    df_two_sum(d[ip], d[ip + 1], s[k].s, s[k].c);
+    df_two_sum(d[ip], -d[ip + 1], a[k].s, a[k].c);
   });
-  auto v = [](const FF& f) {
+  const HeatMoments<FF> f = heat_moments<L, FF>(FF{d[0], 0.f}, s, a);
+  HeatMoments<DF> h;
+  auto v = [](const FF& x) {
     DF r;
-    df_two_sum(f.s, f.c, r.hi, r.lo);
+    df_two_sum(x.s, x.c, r.hi, r.lo);
     return r;
   };
-  m0 = v(f0);
-  for (int a = 0; a < 3; ++a) {
-    m1[a] = v(f1[a]);
-    m3[a] = v(f3[a]);
+  h.m0 = v(f.m0);
+  for (int k = 0; k < L::D; ++k) {
+    h.m1[k] = v(f.m1[k]);
+    h.m3[k] = v(f.m3[k]);
   }
-  for (int c = 0; c < 6; ++c) m2[c] = v(f2[c]);
+  for (int k = 0; k < 6; ++k)
+    if (L::D == 3 || k == 0 || k == 1 || k == 3) h.m2[k] = v(f.m2[k]);
+  return h;
 }
 
 __device__ __forceinline__ double out_double(double x) { return x; }
@@ -920,74 +941,87 @@ __device__ __forceinline__ double out_double(DF x) { return df_to_double(x); }
 // whose FP64 combination ran at the FP64 units' rate; each output is one
 // rounding to double.
 template <class L, class R>
-__device__ __forceinline__ void write_moments(R m0, const R (&m1)[3], const R (&m2)[6], const R (&m3)[3],
-                                              const R (&g)[3], int site, size_t N, int force_order,
-                                              const StepParams& p, double* __restrict__ rho,
+__device__ __forceinline__ void write_moments(const HeatMoments<R>& h, const R (&g)[3], int site, size_t N,
+                                              int force_order, const StepParams& p, double* __restrict__ rho,
                                               double* __restrict__ u, double* __restrict__ T,
                                               double* __restrict__ q) {
   constexpr int D = L::D;
-  const R c = R(L::c), c2 = R(L::c2);
-  const R r = R(1) + m0, ir = R(1) / r;
-  R J[3], uu[3];
-  for (int a = 0; a < 3; ++a) {
-    J[a] = c * m1[a];  // sum f~ xi = rho u~
-    uu[a] = J[a] * ir + R(0.5) * g[a];
+  // the D = 2 sums have no z terms: float-float arithmetic does not fold zeros
+  auto dot = [](const R* x, const R* y) {
+    R r = x[0] * y[0];
+    for (int a = 1; a < D; ++a) r = fma(x[a], y[a], r);
+    return r;
+  };
+  const R r = R(1) + h.m0, ir = R(1) / r;
+  R J[3], ut[3], uu[3];
+  for (int a = 0; a < D; ++a) {
+    J[a] = cmul(L::c, h.m1[a]);  // sum f~ xi = rho u~
+    ut[a] = J[a] * ir;
+    uu[a] = hmac(g[a], ut[a]);
   }
-  const R k2 = m2[0] + m2[1] + m2[2];
-  const R ut2 = (J[0] * J[0] + J[1] * J[1] + J[2] * J[2]) * ir * ir;
-  const R g2 = g[0] * g[0] + g[1] * g[1] + g[2] * g[2];
-  const R Th = ((c2 * k2 - R(D) * m0) * ir - ut2) * R(1.0 / D) + g2 * R(0.25 / D);
+  R k2 = h.m2[0] + h.m2[1];
+  if (D == 3) k2 = k2 + h.m2[2];
+  const R K = cmul(L::c2, k2);
+  const R g2 = dot(g, g);
+  const R Th = fma(fma(K - kscale<D>(h.m0), ir, -dot(ut, ut)), R(1.0 / D), cmul(0.25 / D, g2));
+  const R th = R(1) + Th;
   if (rho) rho[site] = out_double(r);
-  if (T) T[site] = out_double(R(1) + Th);
+  if (T) T[site] = out_double(th);
   if (u)
     for (int a = 0; a < D; ++a) u[a * N + site] = out_double(uu[a]);
   if (!q) return;
-  const R om = site_omega<R>(p, r, R(1) + Th);
-  const R u2 = uu[0] * uu[0] + uu[1] * uu[1] + uu[2] * uu[2];
-  const R ug = uu[0] * g[0] + uu[1] * g[1] + uu[2] * g[2];
-  const R uJ = uu[0] * J[0] + uu[1] * J[1] + uu[2] * J[2];
-  // sum f~ |c|^2 c with P = c^2 m2 (so sum f~ xi xi = delta + P)
-  R Pm[6], Pu[3];
-  for (int k = 0; k < 6; ++k) Pm[k] = c2 * m2[k];
-  sym_mul<R>(Pm, uu, Pu);
-  const R c3 = R(L::c * L::c2);
+  const R om = site_omega<R>(p, r, th);
+  const R u2 = dot(uu, uu), uJ = dot(uu, J);
+  // with P = c^2 m2 (so sum f~ xi xi = delta + P), sum f~ |c|^2 c_a =
+  //   c^3 m3_a - u_a [D + 2 + tr P - 2 u.J + u^2 rho] - 2 (P u)_a + u^2 J_a
+  constexpr int off[3][3] = {{0, 3, 4}, {3, 1, 5}, {4, 5, 2}};
+  const R B = fma(u2, r, K - kscale<2>(uJ)) + R(D + 2);
   R C3[3];
-  for (int a = 0; a < 3; ++a)
-    C3[a] = c3 * m3[a] - R(D + 2) * uu[a] - uu[a] * (c2 * k2) - R(2) * Pu[a] + R(2) * uu[a] * uJ +
-            u2 * J[a] - u2 * uu[a] * r;
+  for (int a = 0; a < D; ++a) {
+    R mu = h.m2[off[a][0]] * uu[0];
+    for (int b = 1; b < D; ++b) mu = fma(h.m2[off[a][b]], uu[b], mu);
+    C3[a] = fma(u2, J[a], cmac(-2.0 * L::c2, mu, cmul(L::c * L::c2, h.m3[a]) - uu[a] * B));
+  }
   // sum F |c|^2 c
   R FC3[3];
-  const R th = R(1) + Th;
   if (force_order >= 2) {
-    for (int a = 0; a < 3; ++a) FC3[a] = R(D + 2) * r * th * g[a];
+    const R rth = kscale<D + 2>(r * th);
+    for (int a = 0; a < D; ++a) FC3[a] = rth * g[a];
     if (force_order == 3) {
       // S = rho (u u + theta delta) - sigma-bar, sigma-bar = -(1 - om/2) S_st
-      R Sst[6], Sg[3];
-      const R iso = fma(r, Th, m0);
-      const R hr = R(0.5) * r;
-      auto conv = [&](int a, int b) { return hr * (uu[a] * (g[b] - uu[b]) + uu[b] * (g[a] - uu[a])); };
-      Sst[0] = Pm[0] - iso + conv(0, 0);
-      Sst[1] = Pm[1] - iso + conv(1, 1);
-      Sst[2] = D == 3 ? Pm[2] - iso + conv(2, 2) : R(0);
-      Sst[3] = Pm[3] + conv(0, 1);
-      Sst[4] = D == 3 ? Pm[4] + conv(0, 2) : R(0);
-      Sst[5] = D == 3 ? Pm[5] + conv(1, 2) : R(0);
-      sym_mul<R>(Sst, g, Sg);
-      const R kf = R(1) - R(0.5) * om;
-      for (int a = 0; a < 3; ++a) FC3[a] += R(2) * kf * Sg[a];
+      const R iso = fma(r, Th, h.m0), hr = half_of(r), kf2 = R(2) - om;
+      for (int a = 0; a < D; ++a) {
+        R Sg = R(0);
+        for (int b = 0; b < D; ++b) {
+          const R conv = hr * fma(uu[a], g[b] - uu[b], uu[b] * (g[a] - uu[a]));
+          R S = cmac(L::c2, h.m2[off[a][b]], conv);
+          if (a == b) S = S - iso;
+          Sg = fma(S, g[b], Sg);
+        }
+        FC3[a] = fma(kf2, Sg, FC3[a]);
+      }
     }
   } else {
     // S = rho delta; M2 = rho (g u + u g) at order 1, 0 at order 0
-    for (int a = 0; a < 3; ++a) {
-      FC3[a] = R(D + 2) * r * g[a] + R(2) * r * uu[a] * ug + r * u2 * g[a];
-      if (force_order == 1) FC3[a] -= R(2) * r * uu[a] * ug + R(2) * r * (g[a] * u2 + uu[a] * ug);
+    const R ug = dot(uu, g);
+    for (int a = 0; a < D; ++a) {
+      const R rg = r * g[a], ru = kscale<2>(r * uu[a]);
+      FC3[a] = force_order == 1 ? fma(rg, R(D + 2) - u2, -(ru * ug)) : fma(rg, R(D + 2) + u2, ru * ug);
     }
   }
-  const R kq = R(0.5) * (R(1) - R(0.5) * om);
-  for (int a = 0; a < D; ++a) q[a * N + site] = out_double(kq * (C3[a] + R(0.5) * FC3[a]));
+  const R kq = half_of(R(1) - half_of(om));
+  for (int a = 0; a < D; ++a) q[a * N + site] = out_double(kq * hmac(FC3[a], C3[a]));
 }
 
-template <class L, int P>
+// Bound by instruction issue (float storage: compensated sums and a
+// float-float combination) or by the FP64 unit (FP64 storage), not by its
+// bytes (Q populations in, 2 + 2 D doubles out).  GB300, against the sums pair
+// by pair with one instantiation for grids with and without solid sites (146
+// registers; now 80 to 96 for the float codecs): 1024 x 512 FP32 85 -> 53 us,
+// FP64 289 -> 212 us, 96^3 FP32 160 -> 97 us, 512 x 512 x 256 FP16 9.2 -> 5.8 ms.
+// SOLID: the grid has solid sites (an own instantiation: the solid pull runs in
+// double and would set the register count of the float codecs' kernel).
+template <class L, int P, bool SOLID>
 __global__ void __launch_bounds__(128) k_moments(const typename Codec<P>::T* __restrict__ fin,
                                                  double* __restrict__ rho, double* __restrict__ u,
                                                  double* __restrict__ T, double* __restrict__ q,
@@ -999,35 +1033,52 @@ __global__ void __launch_bounds__(128) k_moments(const typename Codec<P>::T* __r
   const int z = D == 3 ? p.a0 + (int)blockIdx.z : 0;
   const int site = (z * p.ny + y) * p.nx + x;
   const size_t N = (size_t)p.N;
-  if (p.solid && p.solid[site]) {  // solid sites report zeros
-    if (rho) rho[site] = 0.0;
-    if (T) T[site] = 0.0;
-    for (int a = 0; a < D; ++a) {
-      if (u) u[a * N + site] = 0.0;
-      if (q) q[a * N + site] = 0.0;
+  if constexpr (SOLID) {
+    if (p.solid[site]) {  // solid sites report zeros
+      if (rho) rho[site] = 0.0;
+      if (T) T[site] = 0.0;
+      for (int a = 0; a < D; ++a) {
+        if (u) u[a * N + site] = 0.0;
+        if (q) q[a * N + site] = 0.0;
+      }
+      return;
     }
-    return;
   }
-  if (P != P_FP64 && !p.solid) {
+  const bool near = near_wall(p, D == 2 ? y : z, D == 2 ? p.ny : p.nz);
+  const int wx0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31);
+  const bool interior = !near && wx0 >= 3 && wx0 + 31 <= p.nx - 4;
+  if constexpr (P != P_FP64 && !SOLID) {
     // float storage: the deviations are exact floats; compensated float-pair
     // sums and a float-float combination, no FP64 arithmetic but the final
     // rounding of each output
     float d[Q];
-    pull<L, P, float>(fin, p, x, y, z, d);
-    DF m0, m1[3], m2[6], m3[3];
-    heat_moments_df<L>(d, m0, m1, m2, m3);
+    if (interior) pull_interior<L, P, float>(fin + site, p, y, z, d);
+    else pull<L, P, float>(fin, p, x, y, z, d);
+    const HeatMoments<DF> h = heat_moments_df<L>(d);
     DF g[3];
     site_force_r<D, DF>(p, x, y, z, site, g);
-    write_moments<L, DF>(m0, m1, m2, m3, g, site, N, force_order, p, rho, u, T, q);
-    return;
+    write_moments<L, DF>(h, g, site, N, force_order, p, rho, u, T, q);
+  } else {
+    double d0, s[(Q - 1) / 2], a[(Q - 1) / 2];
+    if constexpr (SOLID) {
+      double d[Q];
+      pull_solid<L, P, double>(fin, p, x, y, z, site, d);
+      pair_split_dev<L, double>(d, d0, s, a);
+    } else if (!near) {
+      double f[Q];
+      if (interior) pull_interior<L, P, double, LD_HINT, IN_STORED>(fin + site, p, y, z, f);
+      else pull_stored<L, P, double>(fin, p, x, y, z, f);
+      pair_split<L, double>(f, d0, s, a);
+    } else {
+      double d[Q];
+      pull<L, P, double>(fin, p, x, y, z, d);
+      pair_split_dev<L, double>(d, d0, s, a);
+    }
+    const HeatMoments<double> h = heat_moments<L, double>(d0, s, a);
+    double g[3];
+    site_force<D>(p, x, y, z, site, g);
+    write_moments<L, double>(h, g, site, N, force_order, p, rho, u, T, q);
   }
-  double d[Q];
-  if (p.solid) pull_solid<L, P, double>(fin, p, x, y, z, site, d);
-  else pull<L, P, double>(fin, p, x, y, z, d);
-  const HeatMoments<L> h = heat_moments<L>(d);
-  double g[3];
-  site_force<D>(p, x, y, z, site, g);
-  write_moments<L, double>(h.m0, h.m1, h.m2, h.m3, g, site, N, force_order, p, rho, u, T, q);
 }
 
 // ------------------------------------------------------ conservation sums

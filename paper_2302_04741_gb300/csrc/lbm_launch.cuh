@@ -177,9 +177,16 @@ struct Ops {
   static cudaError_t moments(int P, const void* fin, double* rho, double* u, double* T_,
                              double* q, int FO, const StepParams& p, cudaStream_t s) {
     const dim3 g = row_grid<L::D>(p, 128), b(128);
-    if (P == P_FP64) k_moments<L, P_FP64><<<g, b, 0, s>>>((const T<P_FP64>*)fin, rho, u, T_, q, FO, p);
-    else if (P == P_FP32S) k_moments<L, P_FP32S><<<g, b, 0, s>>>((const T<P_FP32S>*)fin, rho, u, T_, q, FO, p);
-    else k_moments<L, P_FP16S><<<g, b, 0, s>>>((const T<P_FP16S>*)fin, rho, u, T_, q, FO, p);
+    if (p.solid) {  // FP64 or FP32
+      if (P == P_FP64) k_moments<L, P_FP64, true><<<g, b, 0, s>>>((const T<P_FP64>*)fin, rho, u, T_, q, FO, p);
+      else k_moments<L, P_FP32S, true><<<g, b, 0, s>>>((const T<P_FP32S>*)fin, rho, u, T_, q, FO, p);
+    } else if (P == P_FP64) {
+      k_moments<L, P_FP64, false><<<g, b, 0, s>>>((const T<P_FP64>*)fin, rho, u, T_, q, FO, p);
+    } else if (P == P_FP32S) {
+      k_moments<L, P_FP32S, false><<<g, b, 0, s>>>((const T<P_FP32S>*)fin, rho, u, T_, q, FO, p);
+    } else {
+      k_moments<L, P_FP16S, false><<<g, b, 0, s>>>((const T<P_FP16S>*)fin, rho, u, T_, q, FO, p);
+    }
     return cudaGetLastError();
   }
 
