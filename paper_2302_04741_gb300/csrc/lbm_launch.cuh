@@ -6,6 +6,7 @@
 
 #include "lbm_async.cuh"
 #include "lbm_batch.cuh"
+#include "lbm_half2.cuh"
 #include "lbm_tma.cuh"
 #include "lbm_wave.cuh"
 
@@ -137,6 +138,16 @@ struct Ops {
         default: return cudaErrorInvalidValue;
       }
 #undef LBM_SOLID_CASE
+      return e != cudaSuccess ? e : cudaGetLastError();
+    }
+    if (P == P_FP16S && FO <= 2 && half2_serves(p)) {
+      const int b = half2_block(p.nx, bx);
+      cfg.blockDim = dim3(b);
+      cfg.gridDim = row_grid<L::D>(p, 2 * b);
+      (L::D == 2 ? cfg.gridDim.y : cfg.gridDim.z) = half2_rows(p.na, p.wall != W_NONE);
+      if (FO == 0) e = cudaLaunchKernelEx(&cfg, k_step_half2<L, 0>, (const __half*)fin, (__half*)fout, p);
+      else if (FO == 1) e = cudaLaunchKernelEx(&cfg, k_step_half2<L, 1>, (const __half*)fin, (__half*)fout, p);
+      else e = cudaLaunchKernelEx(&cfg, k_step_half2<L, 2>, (const __half*)fin, (__half*)fout, p);
       return e != cudaSuccess ? e : cudaGetLastError();
     }
 #define LBM_STEP_CASE(PP, FF)                                                            \
