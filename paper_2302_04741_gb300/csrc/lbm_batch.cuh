@@ -13,18 +13,24 @@
 // results to stepping each grid alone).
 #pragma once
 
+#include <stddef.h>
+
 #include "lbm_async.cuh"
 #include "lbm_kernels.cuh"
 
 namespace lbm {
 
 struct __align__(16) BatchGrid {
-  StepParams p;
   void* f[2];
   int cur;
   int pad[3];
+  StepParams p;
 };
 static_assert(sizeof(BatchGrid) % 16 == 0, "BatchGrid is copied as int4");
+// Bytes of a BatchGrid that a CTA stages: all but the double wall tables, which
+// the float codecs do not read (1.3 of 2.6 KB; a tile of a small grid waits for
+// this copy).
+constexpr int BATCH_STAGED = (int)(offsetof(BatchGrid, p) + offsetof(StepParams, fw) + 15) / 16 * 16;
 
 // header[0] = number of grids, header[1] = number of tiles
 template <class L, int P, int FO, int SPT>
@@ -35,7 +41,8 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
   using T = typename C::T;
   using R = typename C::R;
   // the parameters of the tile's grid, staged in shared memory once per tile
-  __shared__ __align__(16) BatchGrid sg;
+  __shared__ __align__(16) unsigned char sgb[BATCH_STAGED];
+  const BatchGrid& sg = *reinterpret_cast<const BatchGrid*>(sgb);
   const int ngrids = __ldg(header), ntiles = __ldg(header + 1);
   const int bx = blockDim.x, TW = bx * SPT;
   int gcur = -1;
@@ -49,8 +56,8 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
     if (lo != gcur) {  // block-uniform
       __syncthreads();
       const int4* src = reinterpret_cast<const int4*>(grids + lo);
-      int4* dst = reinterpret_cast<int4*>(&sg);
-      for (int w = threadIdx.x; w < (int)(sizeof(BatchGrid) / sizeof(int4)); w += bx) dst[w] = src[w];
+      int4* dst = reinterpret_cast<int4*>(sgb);
+      for (int w = threadIdx.x; w < BATCH_STAGED / (int)sizeof(int4); w += bx) dst[w] = src[w];
       __syncthreads();
       gcur = lo;
     }
@@ -105,7 +112,8 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
   using R = typename C::R;
   constexpr int Q = L::Q, D = L::D;
   extern __shared__ __align__(16) unsigned char sbuf[];  // [2][Q][blockDim.x] of T
-  __shared__ __align__(16) BatchGrid sg[2];
+  __shared__ __align__(16) unsigned char sgb[2][BATCH_STAGED];
+  auto slot_of = [&](int k) -> const BatchGrid& { return *reinterpret_cast<const BatchGrid*>(sgb[k]); };
   const int ngrids = __ldg(header), ntiles = __ldg(header + 1);
   const int bx = blockDim.x, tid = threadIdx.x;
   const int stride = bx * (int)sizeof(T);
@@ -123,8 +131,8 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
   };
   auto load_params = [&](int g, int slot) {
     const int4* src = reinterpret_cast<const int4*>(grids + g);
-    int4* dst = reinterpret_cast<int4*>(&sg[slot]);
-    for (int w = tid; w < (int)(sizeof(BatchGrid) / sizeof(int4)); w += bx) dst[w] = src[w];
+    int4* dst = reinterpret_cast<int4*>(sgb[slot]);
+    for (int w = tid; w < BATCH_STAGED / (int)sizeof(int4); w += bx) dst[w] = src[w];
   };
   // site of this thread in tile t of grid g, and whether its warp can be
   // prefetched (32 sites in one row, no x wrap, no wall)
@@ -150,10 +158,10 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
   __syncthreads();
   int site, x, y, z;
   bool fast;
-  geometry(t, g, sg[0].p, site, x, y, z, fast);
+  geometry(t, g, slot_of(0).p, site, x, y, z, fast);
   {
-    const StepParams& p = sg[0].p;
-    const T* fin = static_cast<const T*>(sg[0].f[(sg[0].cur + k) & 1]);
+    const StepParams& p = slot_of(0).p;
+    const T* fin = static_cast<const T*>(slot_of(0).f[(slot_of(0).cur + k) & 1]);
     if (fast) prefetch_interior<L, P>(fin + site, p, y, z, col0, stride);
   }
   cp_async_commit();
@@ -169,18 +177,18 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
     }
     __syncthreads();
     if (tn < ntiles) {
-      const StepParams& pn = sg[ns].p;
+      const StepParams& pn = slot_of(ns).p;
       geometry(tn, gn, pn, siten, xn, yn, zn, fastn);
-      const T* finn = static_cast<const T*>(sg[ns].f[(sg[ns].cur + k) & 1]);
+      const T* finn = static_cast<const T*>(slot_of(ns).f[(slot_of(ns).cur + k) & 1]);
       if (fastn) prefetch_interior<L, P>(finn + siten, pn, yn, zn, col0 + ns * stage_bytes, stride);
     }
     cp_async_commit();
     cp_async_wait<1>();  // this thread's copies of tile t have landed
-    const StepParams& p = sg[cs].p;
+    const StepParams& p = slot_of(cs).p;
     if (site < p.N) {
-      const int par = (sg[cs].cur + k) & 1;
-      const T* __restrict__ fin = static_cast<const T*>(sg[cs].f[par]);
-      T* __restrict__ fout = static_cast<T*>(sg[cs].f[par ^ 1]);
+      const int par = (slot_of(cs).cur + k) & 1;
+      const T* __restrict__ fin = static_cast<const T*>(slot_of(cs).f[par]);
+      T* __restrict__ fout = static_cast<T*>(slot_of(cs).f[par ^ 1]);
       R d[Q];
       if (fast) {
         const T* sc = reinterpret_cast<const T*>(sbuf + cs * stage_bytes) + tid;

@@ -36,12 +36,6 @@ struct StepParams {
   int gaxis;         // G_SINE: axis of the wave
   double g0[3];      // G_UNIFORM / G_SINE amplitude
   const double* gtab;  // G_SINE: sin(2 pi k / n_axis), k < n_axis; G_FIELD: D*N field
-  // thermal wall, side s = 0 (low) / 1 (high): fw = f0_i(1, 0, T_s), fwd = fw - w,
-  // wallA = -sum over one column's incoming slots of fwd, wall_inv_den = 1 / sum of fw
-  double fw[2][QMAX];
-  double fwd[2][QMAX];
-  double wallA[2];
-  double wall_inv_den[2];
   float h_scale;      // FP16 codec scale s and 1/s
   float h_inv_scale;
   // FP16 codec factors per direction, float(w_i) / s and float(1 / w_i) s
@@ -64,10 +58,23 @@ struct StepParams {
   const float* wall_th_f;
   int l2_evict_first;  // 1: population loads are evict-first in L2 (see ld_pop_policy)
   int storage_probe;   // FP64 codec: round stored deviations to P_FP32S / P_FP16S format (0 off)
+  // float copies of the wall constants (set_wall_floats): converted per site
+  // and slot they ran at the FP64 rate, 28 conversions a site of a wall row
+  float fw_f[2][QMAX];
+  float fwd_f[2][QMAX];
+  float wallA_f[2];
+  float wall_inv_den_f[2];
   // layers of the last axis the per-site kernels visit: a0 .. a0 + na - 1
   // (the whole axis, a0 = 0 and na = n_axis, except on a slab context, whose
   // buffer also holds the ghost layers of its neighbours)
   int a0, na;
+  // thermal wall, side s = 0 (low) / 1 (high): fw = f0_i(1, 0, T_s), fwd = fw - w,
+  // wallA = -sum over one column's incoming slots of fwd, wall_inv_den = 1 / sum of fw.
+  // Last: a batch (float codecs) stages what stands before them.
+  double fw[2][QMAX];
+  double fwd[2][QMAX];
+  double wallA[2];
+  double wall_inv_den[2];
 };
 
 // The parameters a kernel of arithmetic type R reads.
@@ -80,6 +87,10 @@ struct ParamsOf<double> {
   __device__ __forceinline__ static double mu(const StepParams& p) { return p.mu; }
   __device__ __forceinline__ static double g0(const StepParams& p, int a) { return p.g0[a]; }
   __device__ __forceinline__ static double gtab(const StepParams& p, size_t k) { return __ldg(p.gtab + k); }
+  __device__ __forceinline__ static double fw(const StepParams& p, int side, int i) { return p.fw[side][i]; }
+  __device__ __forceinline__ static double fwd(const StepParams& p, int side, int i) { return p.fwd[side][i]; }
+  __device__ __forceinline__ static double wallA(const StepParams& p, int side) { return p.wallA[side]; }
+  __device__ __forceinline__ static double wall_inv_den(const StepParams& p, int side) { return p.wall_inv_den[side]; }
 };
 template <>
 struct ParamsOf<float> {
@@ -88,6 +99,10 @@ struct ParamsOf<float> {
   __device__ __forceinline__ static float mu(const StepParams& p) { return p.mu_f; }
   __device__ __forceinline__ static float g0(const StepParams& p, int a) { return p.g0_f[a]; }
   __device__ __forceinline__ static float gtab(const StepParams& p, size_t k) { return __ldg(p.gtab_f + k); }
+  __device__ __forceinline__ static float fw(const StepParams& p, int side, int i) { return p.fw_f[side][i]; }
+  __device__ __forceinline__ static float fwd(const StepParams& p, int side, int i) { return p.fwd_f[side][i]; }
+  __device__ __forceinline__ static float wallA(const StepParams& p, int side) { return p.wallA_f[side]; }
+  __device__ __forceinline__ static float wall_inv_den(const StepParams& p, int side) { return p.wall_inv_den_f[side]; }
 };
 
 template <>
@@ -97,6 +112,10 @@ struct ParamsOf<DF> {
   __device__ __forceinline__ static DF mu(const StepParams& p) { return df_split(p.mu); }
   __device__ __forceinline__ static DF g0(const StepParams& p, int a) { return df_split(p.g0[a]); }
   __device__ __forceinline__ static DF gtab(const StepParams& p, size_t k) { return df_split(__ldg(p.gtab + k)); }
+  __device__ __forceinline__ static DF fw(const StepParams& p, int side, int i) { return df_split(p.fw[side][i]); }
+  __device__ __forceinline__ static DF fwd(const StepParams& p, int side, int i) { return df_split(p.fwd[side][i]); }
+  __device__ __forceinline__ static DF wallA(const StepParams& p, int side) { return df_split(p.wallA[side]); }
+  __device__ __forceinline__ static DF wall_inv_den(const StepParams& p, int side) { return df_split(p.wall_inv_den[side]); }
 };
 
 // ---------------------------------------------------------------- helpers
@@ -336,6 +355,18 @@ template <class L, int P, int I, bool SC>
 __device__ __forceinline__ typename Codec<P>::T step_out(typename Codec<P>::R x, const StepParams& p) {
   if constexpr (SC) return __float2half_rn(x);
   else return Codec<P>::template encode<L, I>(x, p);
+}
+
+// The float copies of the wall constants (host side).
+inline void set_wall_floats(StepParams& p) {
+  for (int side = 0; side < 2; ++side) {
+    for (int i = 0; i < QMAX; ++i) {
+      p.fw_f[side][i] = (float)p.fw[side][i];
+      p.fwd_f[side][i] = (float)p.fwd[side][i];
+    }
+    p.wallA_f[side] = (float)p.wallA[side];
+    p.wall_inv_den_f[side] = (float)p.wall_inv_den[side];
+  }
 }
 
 // The FP16 factors of a lattice for the scale in p (host side).  Both are

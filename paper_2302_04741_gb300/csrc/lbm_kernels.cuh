@@ -149,7 +149,7 @@ __device__ __forceinline__ void pull(const typename Codec<P>::T* __restrict__ fi
         }
       });
     }
-    rm1 = (RR(p.wallA[side]) + sum) * RR(p.wall_inv_den[side]);
+    rm1 = (ParamsOf<RR>::wallA(p, side) + sum) * ParamsOf<RR>::wall_inv_den(p, side);
   }
   static_for<0, Q>([&](auto I) {
     constexpr int i = I;
@@ -165,7 +165,7 @@ __device__ __forceinline__ void pull(const typename Codec<P>::T* __restrict__ fi
       const int mA = side == 0 ? eA - 1 - a : 2 * nA - 1 - sA;
       d[i] = RR(step_in<L, P, io, SC>(ldpop<C, LD>(fin + io * N + colbase + mA * lineA, p), p));
     } else {
-      d[i] = step_from_dev<i, SC>(fma(rm1, RR(p.fw[side][i]), RR(p.fwd[side][i])), p);
+      d[i] = step_from_dev<i, SC>(fma(rm1, ParamsOf<RR>::fw(p, side, i), ParamsOf<RR>::fwd(p, side, i)), p);
     }
   });
 }

@@ -97,6 +97,7 @@ inline void wall_tables(StepParams& p, double T_lo, double T_hi) {
     p.wallA[side] = -sfwd;
     p.wall_inv_den[side] = 1.0 / sfw;
   }
+  set_wall_floats(p);
 }
 
 // Per-site launch: blocks of bx sites along x, one row per block, over the

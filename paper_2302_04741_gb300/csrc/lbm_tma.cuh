@@ -145,7 +145,7 @@ __device__ __forceinline__ void pull_staged(const unsigned char* stage,
         }
       });
     }
-    rm1 = (R(p.wallA[side]) + sum) * R(p.wall_inv_den[side]);
+    rm1 = (ParamsOf<R>::wallA(p, side) + sum) * ParamsOf<R>::wall_inv_den(p, side);
   }
   static_for<0, Q>([&](auto I) {
     constexpr int i = I;
@@ -167,7 +167,7 @@ __device__ __forceinline__ void pull_staged(const unsigned char* stage,
       const int mA = side == 0 ? eA - 1 - a : 2 * nA - 1 - sA;
       d[i] = R(step_in<L, P, io, SC>(C::load(fin + io * N + colbase + mA * lineA, p), p));
     } else {
-      d[i] = step_from_dev<i, SC>(fma(rm1, R(p.fw[side][i]), R(p.fwd[side][i])), p);
+      d[i] = step_from_dev<i, SC>(fma(rm1, ParamsOf<R>::fw(p, side, i), ParamsOf<R>::fwd(p, side, i)), p);
     }
   });
 }
