@@ -64,6 +64,9 @@ struct StepParams {
   float fwd_f[2][QMAX];
   float wallA_f[2];
   float wall_inv_den_f[2];
+  // lanes per site of the FP64 step on a small D2Q37 grid (lbm_split.cuh), 0: one
+  // thread per site; chosen for the whole grid, so that its slabs step alike
+  int split;
   // layers of the last axis the per-site kernels visit: a0 .. a0 + na - 1
   // (the whole axis, a0 = 0 and na = n_axis, except on a slab context, whose
   // buffer also holds the ghost layers of its neighbours)

@@ -7,6 +7,7 @@
 #include "lbm_async.cuh"
 #include "lbm_batch.cuh"
 #include "lbm_half2.cuh"
+#include "lbm_split.cuh"
 #include "lbm_tma.cuh"
 #include "lbm_wave.cuh"
 
@@ -140,6 +141,23 @@ struct Ops {
       }
 #undef LBM_SOLID_CASE
       return e != cudaSuccess ? e : cudaGetLastError();
+    }
+    if constexpr (std::is_same<L, D2Q37>::value) {
+      if (P == P_FP64 && p.split && !p.storage_probe) {
+        cfg.blockDim = dim3(SPLIT_THREADS);
+        cfg.gridDim = dim3(split_blocks(p, p.split));
+#define LBM_SPLIT_CASE(FF)                                                                                          \
+  case FF:                                                                                                          \
+    e = p.split == 2 ? cudaLaunchKernelEx(&cfg, k_step_sym<FF>, (const double*)fin, (double*)fout, p)               \
+                     : cudaLaunchKernelEx(&cfg, k_step_split<FF, 8>, (const double*)fin, (double*)fout, p);         \
+    break;
+        switch (FO) {
+          LBM_SPLIT_CASE(0) LBM_SPLIT_CASE(1) LBM_SPLIT_CASE(2) LBM_SPLIT_CASE(3)
+          default: return cudaErrorInvalidValue;
+        }
+#undef LBM_SPLIT_CASE
+        return e != cudaSuccess ? e : cudaGetLastError();
+      }
     }
     if (P == P_FP16S && FO <= 2 && half2_serves(p)) {
       const int b = half2_block(p.nx, bx);

@@ -30,14 +30,16 @@ def built():
     oracle.set_threads(os.cpu_count() or 1)
 
 
-# one row wider than a warp and its wrap, rows at and between walls
-GRIDS = [(0, (71, 13, 1)), (1, (71, 7, 9))]
+# one row wider than a warp and its wrap, rows at and between walls; the D2Q37
+# grids also span the step's lanes per site (8 up to 608 sites, 2 up to 9,728,
+# then one thread per site), with sites that do not fill the last warp
+GRIDS = [(0, (3, 150, 1)), (0, (13, 7, 1)), (0, (71, 13, 1)), (0, (101, 96, 1)), (0, (101, 99, 1)), (1, (71, 7, 9))]
 
 
 @pytest.mark.parametrize("arith", [0, 1], ids=["double", "pair"])
 @pytest.mark.parametrize("order,sigma", [(0, False), (1, False), (2, False), (2, True)])
 @pytest.mark.parametrize("wall", [0, 1, 2], ids=["periodic", "bounce", "thermal"])
-@pytest.mark.parametrize("lat,shape", GRIDS, ids=["d2", "d3"])
+@pytest.mark.parametrize("lat,shape", GRIDS, ids=["x".join(map(str, s)) for _, s in GRIDS])
 def test_strong_flow(lat, shape, wall, order, sigma, arith):
     D = W.dims(lat)
     g = {"kind": W.G_UNIFORM, "g0": (0.03, -0.05, 0.02 if D == 3 else 0.0)}
@@ -52,6 +54,26 @@ def test_strong_flow(lat, shape, wall, order, sigma, arith):
     ref.step(3)
     far = np.abs(sim.populations() - ref.pulled()[perm_to_oracle(lat)])
     assert far.max() < TOL[arith]
+
+
+@pytest.mark.parametrize("lat,shape", GRIDS[:5], ids=["x".join(map(str, s)) for _, s in GRIDS[:5]])
+@pytest.mark.parametrize("force", ["mu", "sine", "field"])
+@pytest.mark.parametrize("wall", [0, 2], ids=["periodic", "thermal"])
+def test_forces_and_constant_viscosity(lat, shape, wall, force):
+    N = shape[0] * shape[1]
+    g = {"kind": W.G_SINE, "g0": (0.03, -0.02, 0.0), "wave_axis": 0}
+    if force == "field":
+        g = {"kind": W.G_FIELD, "field": 0.05 * (W.uniform(9, 30, 2 * N).reshape(2, N) - 0.5)}
+    w = workload(lat, shape, tau=0.7, g=g, bc=(0, wall, 0))
+    w["T_lo"], w["T_hi"] = (1.0, 1.15, 1.0), (1.0, 0.9, 1.0)
+    w["rho"], w["u"], w["T"] = smooth_state(lat, shape, 12, amp_u=0.3, amp_T=0.2, amp_rho=0.2)
+    if force == "mu":
+        w["mu"] = 0.2
+    sim, ref = lbm.Sim(w, graph_steps=2).init(), oracle_sim(w)
+    sim.step(3)
+    ref.step(3)
+    far = np.abs(sim.populations() - ref.pulled()[perm_to_oracle(lat)])
+    assert far.max() < TOL[0]
 
 
 @pytest.mark.parametrize("arith", [0, 1], ids=["double", "pair"])
