@@ -101,6 +101,68 @@ __device__ __forceinline__ bool near_wall(const StepParams& p, int a, int nA) {
   return p.wall != W_NONE && (a < 3 || a >= nA - 3);
 }
 
+// sum + the deviation of a stored value of wall row ROW, in the sum of a thermal
+// wall.  FP16 storage: the decode's product is fused into the sum, but for the
+// row-2 population of D3Q39 (0, 0, +-3), which is rounded first (written out, so
+// that every kernel forms the same wall density).
+template <class L, int P, int J, int ROW, class RR>
+__device__ __forceinline__ RR add_deviation(RR sum, typename Codec<P>::T v, const StepParams& p) {
+  if constexpr (P == P_FP16S && std::is_same<RR, float>::value) {
+    if constexpr (L::D == 3 && ROW == 2) return __fadd_rn(sum, __fmul_rn(__half2float(v), p.h_dec[J]));
+    else return fmaf(__half2float(v), p.h_dec[J], sum);
+  } else {
+    return sum + RR(Codec<P>::template decode<L, J>(v, p));
+  }
+}
+
+// Pull of a site in one of the three rows next to the wall on side SIDE: slots
+// whose source lies beyond it follow the wall rule.  The side is a template
+// parameter: the populations that leave the column through the wall (26 on
+// D2Q37) are then a fixed list, loaded without a predicate each.
+template <class L, int P, class RR, int LD, bool SC, int SIDE>
+__device__ __forceinline__ void pull_near(const typename Codec<P>::T* __restrict__ fin, const StepParams& p, int x, int y,
+                                          int z, int a, int nA, const int (&xs)[7], const int (&ys)[7],
+                                          const int (&zs)[7], RR (&d)[L::Q]) {
+  using C = Codec<P>;
+  constexpr int D = L::D, Q = L::Q;
+  const int nx = p.nx, ny = p.ny;
+  const size_t N = (size_t)p.N;
+  const int colbase = D == 2 ? x : (y * nx + x);     // site of the column at wall coord 0
+  const int lineA = D == 2 ? nx : nx * ny;           // stride along the wall axis
+  RR rm1 = RR(0);                                    // rho_w - 1 of the thermal wall
+  if (p.wall == W_THERMAL) {
+    RR sum = RR(0);
+    static_for<0, 3>([&](auto ROW) {
+      constexpr int r = ROW;
+      const int row = SIDE == 0 ? r : nA - 1 - r;
+      static_for<0, Q>([&](auto J) {
+        constexpr int j = J;
+        constexpr int eA = L::E(j, D - 1);
+        if constexpr (SIDE == 0 ? eA < 0 && r + eA < 0 : eA > 0 && r - eA < 0)
+          sum = add_deviation<L, P, j, r>(sum, ldpop<C, LD>(fin + j * N + colbase + row * lineA, p), p);
+      });
+    });
+    rm1 = (ParamsOf<RR>::wallA(p, SIDE) + sum) * ParamsOf<RR>::wall_inv_den(p, SIDE);
+  }
+  static_for<0, Q>([&](auto I) {
+    constexpr int i = I;
+    constexpr int ex = L::E(i, 0), ey = L::E(i, 1), ez = L::E(i, 2);
+    constexpr int eA = L::E(i, D - 1);
+    const int sA = a - eA;
+    if ((SIDE == 0 ? eA <= 0 : eA >= 0) || (SIDE == 0 ? sA >= 0 : sA < nA)) {
+      const int off = zs[ez + 3] + ys[ey + 3] + xs[ex + 3];
+      d[i] = RR(step_in<L, P, i, SC>(ldpop<C, LD>(fin + i * N + off, p), p));
+    } else if (p.wall == W_BOUNCE) {
+      // d_i = d_io and w_i = w_io: the scaled values agree as well
+      constexpr int io = opposite<i>();
+      const int mA = SIDE == 0 ? eA - 1 - a : 2 * nA - 1 - sA;
+      d[i] = RR(step_in<L, P, io, SC>(ldpop<C, LD>(fin + io * N + colbase + mA * lineA, p), p));
+    } else {
+      d[i] = step_from_dev<i, SC>(fma(rm1, ParamsOf<RR>::fw(p, SIDE, i), ParamsOf<RR>::fwd(p, SIDE, i)), p);
+    }
+  });
+}
+
 // Pull of all Q populations of site (x, y, z) with the boundary rules, decoded
 // to deviations in type RR (SC: the scaled values of an FP16-scaled step, see
 // scaled_step).  The wall axis is the last axis (y in 2-D, z in 3-D).
@@ -129,45 +191,9 @@ __device__ __forceinline__ void pull(const typename Codec<P>::T* __restrict__ fi
     });
     return;
   }
-  // ---- a row next to a wall: slots whose source lies beyond the wall
-  const int side = a < 3 ? 0 : 1;
-  const int colbase = D == 2 ? x : (y * nx + x);     // site of the column at wall coord 0
-  const int lineA = D == 2 ? nx : nx * ny;           // stride along the wall axis
-  RR rm1 = RR(0);                                    // rho_w - 1 of the thermal wall
-  if (p.wall == W_THERMAL) {
-    RR sum = RR(0);
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-      const int row = side == 0 ? r : nA - 1 - r;
-      static_for<0, Q>([&](auto J) {
-        constexpr int j = J;
-        constexpr int eA = L::E(j, D - 1);
-        if constexpr (eA != 0) {
-          const bool leaves = side == 0 ? (eA < 0 && r + eA < 0) : (eA > 0 && r - eA < 0);
-          if (leaves)
-            sum += RR(C::template decode<L, j>(ldpop<C, LD>(fin + j * N + colbase + row * lineA, p), p));
-        }
-      });
-    }
-    rm1 = (ParamsOf<RR>::wallA(p, side) + sum) * ParamsOf<RR>::wall_inv_den(p, side);
-  }
-  static_for<0, Q>([&](auto I) {
-    constexpr int i = I;
-    constexpr int ex = L::E(i, 0), ey = L::E(i, 1), ez = L::E(i, 2);
-    constexpr int eA = L::E(i, D - 1);
-    const int sA = a - eA;
-    if (sA >= 0 && sA < nA) {
-      const int off = zs[ez + 3] + ys[ey + 3] + xs[ex + 3];
-      d[i] = RR(step_in<L, P, i, SC>(ldpop<C, LD>(fin + i * N + off, p), p));
-    } else if (p.wall == W_BOUNCE) {
-      // d_i = d_io and w_i = w_io: the scaled values agree as well
-      constexpr int io = opposite<i>();
-      const int mA = side == 0 ? eA - 1 - a : 2 * nA - 1 - sA;
-      d[i] = RR(step_in<L, P, io, SC>(ldpop<C, LD>(fin + io * N + colbase + mA * lineA, p), p));
-    } else {
-      d[i] = step_from_dev<i, SC>(fma(rm1, ParamsOf<RR>::fw(p, side, i), ParamsOf<RR>::fwd(p, side, i)), p);
-    }
-  });
+  // a row next to a wall (block-uniform side)
+  if (a < 3) pull_near<L, P, RR, LD, SC, 0>(fin, p, x, y, z, a, nA, xs, ys, zs, d);
+  else pull_near<L, P, RR, LD, SC, 1>(fin, p, x, y, z, a, nA, xs, ys, zs, d);
 }
 
 // ------------------------------------------------------- solid sites
