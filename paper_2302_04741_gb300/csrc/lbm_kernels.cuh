@@ -1112,7 +1112,7 @@ __global__ void __launch_bounds__(128) k_moments(const typename Codec<P>::T* __r
 // the exact sum is s + c up to the rounding of c.
 template <class R>
 struct RSum {
-  R s = R(0), c = R(0);
+  R s, c;
   __device__ __forceinline__ void add(R v) {
     const R t = s + v;
     c += fabs(s) >= fabs(v) ? (s - t) + v : (v - t) + s;
@@ -1132,56 +1132,52 @@ constexpr int NCONS = 5;
 // slot, then the block's number of fluid sites (a double at index 2 NCONS).
 constexpr int CONS_SLOT = 2 * NCONS + 1;
 
-// Block-wide merge of per-thread compensated pairs in a fixed order: the
-// pairs go to shared memory, 8 threads per quantity merge contiguous runs of
-// BS / 8, thread 0 merges the 8 runs; the counts are summed by warp shuffles.
-// All in R: with float storage no FP64 instruction runs here (GB300 issues
-// FP64 at a small fraction of the FP32 rate, so a double-precision tree at
-// the end of every block was the tail of the pass).  The totals are valid in
-// thread 0 only.
-template <class R, int BS>
+// Block-wide merge of per-thread compensated pairs in a fixed order: the pairs
+// go to shared memory, one warp merges a quantity (each lane BS / 32 threads'
+// pairs, then five shuffle steps), so a block's merge is BS / 32 + 4 dependent
+// merges long.  All in R: with float storage no FP64 instruction runs here, with
+// FP64 storage a merge is six of them at 64 cycles each, and this chain (of the
+// blocks, and again of the last one) was most of a small grid's pass.  `tot`
+// (shared memory) and the counts are valid in every thread afterwards; z is
+// left out on two-dimensional grids.
+template <class R, int BS, int D>
 __device__ __forceinline__ void reduce_block(const RSum<R> (&v)[NCONS], unsigned n, unsigned bad,
                                              RSum<R> (&tot)[NCONS], unsigned& ntot,
                                              unsigned& btot) {
   static_assert(BS % 32 == 0 && BS >= 64, "block size");
-  constexpr int RUN = BS / 8;
   __shared__ R sh_s[NCONS][BS], sh_c[NCONS][BS];
-  __shared__ RSum<R> sh_p[NCONS][8];
   __shared__ unsigned sh_n[BS / 32], sh_b[BS / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int k = 0; k < NCONS; ++k) {
+    if (D == 2 && k == 3) continue;
     sh_s[k][tid] = v[k].s;
     sh_c[k][tid] = v[k].c;
   }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    n += __shfl_down_sync(0xffffffffu, n, off);
-    bad += __shfl_down_sync(0xffffffffu, bad, off);
-  }
+  n = __reduce_add_sync(0xffffffffu, n);
+  bad = __reduce_add_sync(0xffffffffu, bad);
   if (lane == 0) {
     sh_n[warp] = n;
     sh_b[warp] = bad;
   }
   __syncthreads();
-  if (tid < NCONS * 8) {
-    const int k = tid / 8, r = tid % 8;
-    RSum<R> a{sh_s[k][r * RUN], sh_c[k][r * RUN]};
-    for (int j = 1; j < RUN; ++j) a.merge(RSum<R>{sh_s[k][r * RUN + j], sh_c[k][r * RUN + j]});
-    sh_p[k][r] = a;
+  constexpr int NK = D == 2 ? NCONS - 1 : NCONS;
+  for (int q = warp; q < NK; q += BS / 32) {
+    const int k = D == 2 && q == 3 ? 4 : q;
+    RSum<R> a{sh_s[k][lane], sh_c[k][lane]};
+#pragma unroll
+    for (int j = 1; j < BS / 32; ++j) a.merge(RSum<R>{sh_s[k][lane + 32 * j], sh_c[k][lane + 32 * j]});
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+      a.merge(RSum<R>{__shfl_down_sync(0xffffffffu, a.s, off), __shfl_down_sync(0xffffffffu, a.c, off)});
+    if (lane == 0) tot[k] = a;
   }
+  if (D == 2 && tid == 0) tot[3] = RSum<R>{};
   __syncthreads();
-  if (tid == 0) {
-    for (int k = 0; k < NCONS; ++k) {
-      RSum<R> a = sh_p[k][0];
-      for (int r = 1; r < 8; ++r) a.merge(sh_p[k][r]);
-      tot[k] = a;
-    }
-    ntot = 0u;
-    btot = 0u;
-    for (int w = 0; w < BS / 32; ++w) {
-      ntot += sh_n[w];
-      btot += sh_b[w];
-    }
+  ntot = 0u;
+  btot = 0u;
+  for (int w = 0; w < BS / 32; ++w) {
+    ntot += sh_n[w];
+    btot += sh_b[w];
   }
 }
 
@@ -1228,7 +1224,7 @@ template <class L, class R, int BS>
 __device__ __forceinline__ void reduce_partials(const double* __restrict__ part,
                                                 const unsigned* __restrict__ badcount, int nblocks,
                                                 const StepParams& p, double* out) {
-  RSum<R> f[NCONS];
+  RSum<R> f[NCONS] = {};
   unsigned n = 0u, b = 0u;
   for (int blk = threadIdx.x; blk < nblocks; blk += BS) {
     const double* slot = part + (size_t)blk * CONS_SLOT;
@@ -1237,9 +1233,9 @@ __device__ __forceinline__ void reduce_partials(const double* __restrict__ part,
     n += (unsigned)__ldcg(slot + 2 * NCONS);
     b += __ldcg(badcount + blk);
   }
-  RSum<R> tot[NCONS];
+  __shared__ RSum<R> tot[NCONS];
   unsigned ntot, btot;
-  reduce_block<R, BS>(f, n, b, tot, ntot, btot);
+  reduce_block<R, BS, L::D>(f, n, b, tot, ntot, btot);
   if (threadIdx.x == 0) {
     conserved_from_sums<L, R>(tot, double(ntot), p, out);
     out[2 * NCONS] = double(btot);
@@ -1281,7 +1277,7 @@ __global__ void __launch_bounds__(128, LBM_CONSERVED_BLOCKS) k_conserved(const t
   const int ntx = (p.nx + 127) / 128;
   const int ntiles = ntx * (D == 2 ? p.na : p.ny * p.na);
   const bool uniform = p.gkind == G_UNIFORM;
-  RSum<R> sums[NCONS];
+  RSum<R> sums[NCONS] = {};
   unsigned count = 0u, bad = 0u;
   const bool walls = p.wall != W_NONE;
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
@@ -1294,14 +1290,33 @@ __global__ void __launch_bounds__(128, LBM_CONSERVED_BLOCKS) k_conserved(const t
     if (x >= p.nx) continue;
     const int site = (z * p.ny + y) * p.nx + x;
     if (p.solid && p.solid[site]) continue;
-    R d[Q];
     const int a = D == 2 ? y : z;
     const int nA = D == 2 ? p.ny : p.nz;
     const int wx0 = xt * 128 + (threadIdx.x & ~31);
-    const bool interior = !(walls && (a < 3 || a >= nA - 3)) && wx0 >= 3 && wx0 + 31 <= p.nx - 4;
-    if (p.solid) pull_solid<L, P, R>(fin, p, x, y, z, site, d);
-    else if (interior) pull_interior<L, P, R>(fin + site, p, y, z, d);
-    else pull<L, P, R>(fin, p, x, y, z, d);
+    const bool near = near_wall(p, a, nA);
+    const bool interior = !near && wx0 >= 3 && wx0 + 31 <= p.nx - 4;
+    RawMoments<L, R> r;
+    if constexpr (P == P_FP64) {  // pair sums and mirror groups: fewer FP64 operations
+      R d0, s[(Q - 1) / 2], am[(Q - 1) / 2];
+      if (!p.solid && !near) {
+        R f[Q];
+        if (interior) pull_interior<L, P, R, LD_HINT, IN_STORED>(fin + site, p, y, z, f);
+        else pull_stored<L, P, R>(fin, p, x, y, z, f);
+        pair_split<L, R>(f, d0, s, am);
+      } else {
+        R d[Q];
+        if (p.solid) pull_solid<L, P, R>(fin, p, x, y, z, site, d);
+        else pull<L, P, R>(fin, p, x, y, z, d);
+        pair_split_dev<L, R>(d, d0, s, am);
+      }
+      r = pair_moments<L, R>(d0, s, am);
+    } else {
+      R d[Q];
+      if (p.solid) pull_solid<L, P, R>(fin, p, x, y, z, site, d);
+      else if (interior) pull_interior<L, P, R>(fin + site, p, y, z, d);
+      else pull<L, P, R>(fin, p, x, y, z, d);
+      r = raw_moments<L, R>(d);
+    }
     R g[3];
     if (sizeof(R) == sizeof(float) && p.gkind == G_FIELD && p.gtab_f == nullptr) {
       // a caller's double field without a float copy (lbm_conserved_static),
@@ -1312,7 +1327,6 @@ __global__ void __launch_bounds__(128, LBM_CONSERVED_BLOCKS) k_conserved(const t
     } else {
       site_force_r<D, R>(p, x, y, z, site, g);
     }
-    const RawMoments<L, R> r = raw_moments<L, R>(d);
     ++count;
     sums[0].add(r.drho);
     const R j0 = mul_c<L, R>(r.j[0]), j1 = mul_c<L, R>(r.j[1]), j2 = mul_c<L, R>(r.j[2]);
@@ -1338,9 +1352,9 @@ __global__ void __launch_bounds__(128, LBM_CONSERVED_BLOCKS) k_conserved(const t
     bad += (rr > R(0) && e > R(0) && isfinite(e)) ? 0u : 1u;
   }
   {
-    RSum<R> tot[NCONS];
+    __shared__ RSum<R> tot[NCONS];
     unsigned ntot, btot;
-    reduce_block<R, 128>(sums, count, bad, tot, ntot, btot);
+    reduce_block<R, 128, D>(sums, count, bad, tot, ntot, btot);
     if (threadIdx.x == 0) {
       double* slot = part + (size_t)blockIdx.x * CONS_SLOT;
       R* rs = reinterpret_cast<R*>(slot);
