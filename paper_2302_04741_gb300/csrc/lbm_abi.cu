@@ -283,9 +283,12 @@ int launch_one_step(lbm_ctx* c) {
   else if (c->use_async)
     e = c->ops->step_async(c->fo, c->f[c->cur], c->f[c->cur ^ 1], c->p, c->async_grid,
                            c->opt.block_x, c->stream);
-  else
+  else {
+    StepParams p = c->p;
+    p.reverse = c->opt.precision == LBM_FP32_SHIFTED ? c->cur : 0;
     e = c->ops->step(c->opt.fp64_arith == LBM_ARITH_FLOAT_PAIR ? (int)lbm::P_FP64DF : c->opt.precision,
-                     c->fo, c->f[c->cur], c->f[c->cur ^ 1], c->p, c->opt.block_x, c->overlap, c->stream);
+                     c->fo, c->f[c->cur], c->f[c->cur ^ 1], p, c->opt.block_x, c->overlap, c->stream);
+  }
   if (e != cudaSuccess) return fail(c, LBM_ECUDA, "step launch failed: %s", cudaGetErrorString(e));
   c->cur ^= 1;
   return LBM_OK;

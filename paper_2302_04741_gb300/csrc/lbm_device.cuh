@@ -57,6 +57,7 @@ struct StepParams {
   const double* wall_th;
   const float* wall_th_f;
   int l2_evict_first;  // 1: population loads are evict-first in L2 (see ld_pop_policy)
+  int reverse;         // 1: the launch visits the lines of the grid in descending order (launch_line)
   int storage_probe;   // FP64 codec: round stored deviations to P_FP32S / P_FP16S format (0 off)
   // float copies of the wall constants (set_wall_floats): converted per site
   // and slot they ran at the FP64 rate, 28 conversions a site of a wall row
@@ -225,8 +226,16 @@ __device__ __forceinline__ R edot(const R (&v)[3]) {
 // launches under a profiler showed no gain (the same DRAM reads, fewer
 // writes inside the launch), so the benefit comes from how consecutive steps
 // share L2 and DRAM.  On working sets of twice L2 and more the hint cost
-// 4-8 %, so the host sets the flag only below 1.5 times the L2 size.  The
-// results are bit-identical either way.
+// 4-8 %, so the host sets the flag only below 1.5 times the L2 size.
+// FP32 steps alternate the direction in which they visit the lines of the grid
+// (StepParams::reverse): the lines written last, which L2 still holds, are read
+// first.  Microseconds a step, ascending -> alternating: 1024 x 512 22.15 ->
+// 21.68, 1024 x 700 (1.6 times L2) 33.7 -> 31.7, 96^3 (2.1 times) 42.8 -> 41.1,
+// 1400 x 900 (2.9 times) 57.2 -> 55.5, 256^2 x 128 (20 times) the same.  (With
+// the hint up to 2.25 times L2 the middle two took 30.7 and 40.6, but three 96^3
+// boxes stepped at once 4 % longer than without.)  The two-site FP16 step
+// gained nothing (1024 x 512 14.7 -> 16.3), nor did a batch in reversed tile
+// order.  The results are bit-identical either way.
 template <class T>
 __device__ __forceinline__ T ld_pop_policy(const T* ptr, bool evict_first) {
   unsigned long long first, normal;

@@ -551,6 +551,11 @@ __device__ __forceinline__ int wall_rows_first(int b, int n, bool walls) {
   if (!walls || n < 6) return b;
   return b < 3 ? b : (b < 6 ? n - 6 + b : b - 3);
 }
+// The same with the bulk lines in the launch's direction (StepParams::reverse).
+__device__ __forceinline__ int launch_line(int b, int n, bool walls, int reverse) {
+  if (!walls || n < 6) return reverse ? n - 1 - b : b;
+  return b < 3 ? b : (b < 6 ? n - 6 + b : (reverse ? n + 2 - b : b - 3));
+}
 
 // SOLID: the grid has solid sites (they are skipped; their fluid neighbours
 // take the diffuse-wall pull).
@@ -562,8 +567,9 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= p.nx) return;
   const bool walls = p.wall != W_NONE;
-  const int y = L::D == 2 ? p.a0 + wall_rows_first(blockIdx.y, p.na, walls) : (int)blockIdx.y;
-  const int z = L::D == 3 ? p.a0 + wall_rows_first(blockIdx.z, p.na, walls) : (int)blockIdx.z;
+  const int y = L::D == 2 ? p.a0 + launch_line(blockIdx.y, p.na, walls, p.reverse)
+                          : (p.reverse ? p.ny - 1 - (int)blockIdx.y : (int)blockIdx.y);
+  const int z = L::D == 3 ? p.a0 + launch_line(blockIdx.z, p.na, walls, p.reverse) : 0;
   const int site = (z * p.ny + y) * p.nx + x;
   if constexpr (SOLID) {
     if (__ldg(p.solid + site)) return;
