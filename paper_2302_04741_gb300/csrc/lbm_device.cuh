@@ -351,12 +351,6 @@ __device__ __forceinline__ typename Codec<P>::R step_in(typename Codec<P>::T v, 
   if constexpr (SC) return __half2float(v);
   else return Codec<P>::template decode<L, I>(v, p);
 }
-// the stored value of FP64 storage in the step's arithmetic
-template <int P>
-__device__ __forceinline__ typename Codec<P>::R stored_value(double v) {
-  if constexpr (P == P_FP64DF) return df_split(v);
-  else return v;
-}
 // a deviation formed in the kernel (a wall slot) in the working representation
 template <int I, bool SC, class R>
 __device__ __forceinline__ R step_from_dev(R d, const StepParams& p) {

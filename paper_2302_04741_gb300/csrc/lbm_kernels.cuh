@@ -12,6 +12,7 @@
 
 #include "lbm_device.cuh"
 #include "lbm_poly.cuh"
+#include "lbm_df2.cuh"
 
 namespace lbm {
 
@@ -68,7 +69,7 @@ __device__ __forceinline__ void site_force_r(const StepParams& p, int x, int y, 
 enum { IN_DEV = 0, IN_SCALED = 1, IN_STORED = 2 };
 template <class L, int P, int I, int IN>
 __device__ __forceinline__ typename Codec<P>::R pulled_value(typename Codec<P>::T v, const StepParams& p) {
-  if constexpr (IN == IN_STORED) return stored_value<P>(v);
+  if constexpr (IN == IN_STORED) return v;
   else return step_in<L, P, I, IN == IN_SCALED>(v, p);
 }
 
@@ -442,20 +443,13 @@ __device__ __forceinline__ void pair_split_dev(const R (&d)[L::Q], R& d0, R (&s)
   });
 }
 
-// Collision of one site of an FP64 grid (IEEE double or float-float) from its
-// pair sums and differences, and store of f*(x): see lbm_poly.cuh.
-template <class L, int P, int FO>
-__device__ __forceinline__ void poly_store(typename Codec<P>::R d0, const typename Codec<P>::R (&s)[(L::Q - 1) / 2],
-                                           const typename Codec<P>::R (&a)[(L::Q - 1) / 2],
-                                           const typename Codec<P>::R (&g)[3], int site,
-                                           typename Codec<P>::T* __restrict__ fout, const StepParams& p) {
-  using C = Codec<P>;
-  using R = typename C::R;
+// The mid-point state of an FP64 site (R1: rho, u = u~ + g/2, theta) from its raw
+// moments, and the polynomial's coefficients.  stress(m, u, S): the tensor S of
+// the sigma-bar terms (FO 3).
+template <class L, class R, int FO, class K, class STRESS>
+__device__ __forceinline__ void site_coefficients(const RawMoments<L, R>& r, const R (&g)[3], const StepParams& p,
+                                                  SiteState<R>& m, K& k, STRESS&& stress) {
   constexpr int D = L::D;
-  const size_t N = (size_t)p.N;
-  const RawMoments<L, R> r = pair_moments<L, R>(d0, s, a);
-  // mid-point state (R1): rho, u = u~ + g/2, theta
-  SiteState<R> m;
   m.drho = r.drho;
   m.rho = R(1) + r.drho;
   const R irho = R(1) / m.rho;
@@ -473,7 +467,6 @@ __device__ __forceinline__ void poly_store(typename Codec<P>::R d0, const typena
   m.Th = fma(fma(mul_c2<L, R>(r.k2) - kscale<D>(r.drho), irho, -ut2), R(1.0 / D), g2 * R(0.25 / D));
   m.om = site_omega<R>(p, m.rho, R(1) + m.Th);
   m.rom = m.rho * m.om;
-  const R om1 = R(1) - m.om, hom1 = half_of(om1);
   const R rk = m.rho - half_of(m.rom);
   m.rkgu = FO >= 1 ? rk * gu : R(0);
   m.T = mul_c2<L, R>(m.Th);
@@ -482,29 +475,72 @@ __device__ __forceinline__ void poly_store(typename Codec<P>::R d0, const typena
     m.U[c] = c < D ? mul_c<L, R>(u[c]) : R(0);
     m.S[c] = c < D ? crk * g[c] : R(0);
   }
-  typename std::conditional<D == 2, PolyCoef2<R>, PolyCoef3<R>>::type k;
-  poly_coef<(FO == 3 ? 2 : FO)>(m, k);
+  if constexpr (D == 2 && std::is_same<R, DF>::value) poly_coef2<(FO == 3 ? 2 : FO)>(m, k);
+  else poly_coef<(FO == 3 ? 2 : FO)>(m, k);
   if constexpr (FO == 3) {
     R S[6];
-    stress_tensor_pairs<L, R>(s, r.drho, m.rho, m.Th, u, g, S);
+    stress(m, u, S);
     const R kf = R(1) - half_of(m.om);
     poly_add_stress(stress_terms<L, R>(S, g, half_of(kf * kf)), k);
   }
-  typename C::T* __restrict__ fo = fout + site;
+}
+template <class L, class R>
+using PolyCoefOf = typename std::conditional<L::D == 2, PolyCoef2<R>, PolyCoef3<R>>::type;
+
+// Collision of one site of an FP64 grid in IEEE double from its pair sums and
+// differences, and store of f*(x): see lbm_poly.cuh.
+template <class L, int FO>
+__device__ __forceinline__ void poly_store(double d0, const double (&s)[(L::Q - 1) / 2],
+                                           const double (&a)[(L::Q - 1) / 2], const double (&g)[3], int site,
+                                           double* __restrict__ fout, const StepParams& p) {
+  const size_t N = (size_t)p.N;
+  SiteState<double> m;
+  PolyCoefOf<L, double> k;
+  site_coefficients<L, double, FO>(pair_moments<L, double>(d0, s, a), g, p, m, k,
+                                   [&](const SiteState<double>& st, const double (&u)[3], double (&S)[6]) {
+                                     stress_tensor_pairs<L, double>(s, st.drho, st.rho, st.Th, u, g, S);
+                                   });
+  const double om1 = 1.0 - m.om, hom1 = 0.5 * om1;
+  double* __restrict__ fo = fout + site;
   // FP64 storage probe: the stored deviation rounded as a float codec stores it
-  const bool probe = P == P_FP64 && p.storage_probe != 0;
-  auto put = [&](auto I, R d) {
+  const bool probe = p.storage_probe != 0;
+  auto put = [&](auto I, double d) {
     constexpr int i = I;
-    if constexpr (P == P_FP64)
-      if (probe) d = probe_round<i>(d, p);
-    fo[i * N] = C::template encode<L, i>(d, p);
+    if (probe) d = probe_round<i>(d, p);
+    fo[i * N] = Codec<P_FP64>::template encode<L, i>(d, p);
   };
-  put(ic<0>{}, fma(d0, om1, cmul(L::W(0), const_term(k))));
-  poly_pairs<L, R>(k, [&](auto K, R wev, R wod) {
+  put(ic<0>{}, fma(d0, om1, L::W(0) * const_term(k)));
+  poly_pairs<L, double>(k, [&](auto K, double wev, double wod) {
     constexpr int kp = K;
-    const R ev = fma(hom1, s[kp], wev), od = fma(hom1, a[kp], wod);
+    const double ev = fma(hom1, s[kp], wev), od = fma(hom1, a[kp], wod);
     put(ic<2 * kp + 1>{}, ev + od);
     put(ic<2 * kp + 2>{}, ev - od);
+  });
+}
+
+// The same in float-float, the (s, a) of a pair in one pack (lbm_df2.cuh).
+template <class L, int FO>
+__device__ __forceinline__ void df2_store(DF d0, const DF2 (&v)[(L::Q - 1) / 2], const DF (&g)[3], int site,
+                                          double* __restrict__ fout, const StepParams& p) {
+  const size_t N = (size_t)p.N;
+  SiteState<DF> m;
+  PolyCoefOf<L, DF> k;
+  site_coefficients<L, DF, FO>(pair_moments2<L>(d0, v), g, p, m, k,
+                               [&](const SiteState<DF>& st, const DF (&u)[3], DF (&S)[6]) {
+                                 DF s[(L::Q - 1) / 2];
+                                 static_for<0, (L::Q - 1) / 2>([&](auto K) { s[K] = px(v[K]); });
+                                 stress_tensor_pairs<L, DF>(s, st.drho, st.rho, st.Th, u, g, S);
+                               });
+  const DF om1 = DF(1) - m.om;
+  const DF hom1 = half_of(om1);
+  double* __restrict__ fo = fout + site;
+  fo[0] = Codec<P_FP64DF>::template encode<L, 0>(fma(d0, om1, cmul(L::W(0), const_term(k))), p);
+  poly_pairs2<L>(k, [&](auto K, DF2 wg) {
+    constexpr int kp = K;
+    constexpr F2 w = f2_of(L::W(2 * kp + 1));
+    const double2 o = pair_out(hom1, v[kp], wg, w.hi, w.lo);
+    fo[(2 * kp + 1) * N] = o.x;
+    fo[(2 * kp + 2) * N] = o.y;
   });
 }
 
@@ -582,7 +618,7 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
     if constexpr (P == P_FP64) {
       R d0, s[(L::Q - 1) / 2], a[(L::Q - 1) / 2];
       pair_split_dev<L, R>(d, d0, s, a);
-      poly_store<L, P, FO>(d0, s, a, g, site, fout, p);
+      poly_store<L, FO>(d0, s, a, g, site, fout, p);
     } else {
       collide_store<L, P, FO>(d, g, site, fout, p);
     }
@@ -606,7 +642,7 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
     if (interior) pull_interior<L, P, R, LD_HINT, SC ? IN_SCALED : IN_DEV>(fin + site, p, y, z, d);
     else pull<L, P, R, LD_HINT, SC>(fin, p, x, y, z, d);
     collide_store<L, P, FO, SC>(d, g, site, fout, p);
-  } else {
+  } else if constexpr (P == P_FP64) {
     R d0, s[(L::Q - 1) / 2], am[(L::Q - 1) / 2];
     if (!near) {
       R f[L::Q];
@@ -618,7 +654,27 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
       pull<L, P, R>(fin, p, x, y, z, d);
       pair_split_dev<L, R>(d, d0, s, am);
     }
-    poly_store<L, P, FO>(d0, s, am, g, site, fout, p);
+    poly_store<L, FO>(d0, s, am, g, site, fout, p);
+  } else {
+    DF d0;
+    DF2 v[(L::Q - 1) / 2];
+    if (!near) {
+      double f[L::Q];
+      if (interior) pull_interior<L, P_FP64, double, LD_HINT, IN_STORED>(fin + site, p, y, z, f);
+      else pull_stored<L, P_FP64, double>(fin, p, x, y, z, f);
+      d0 = df_split(f[0]) - DF(L::W(0));
+      static_for<0, (L::Q - 1) / 2>([&](auto K) {
+        constexpr int ip = 2 * K + 1;
+        constexpr F2 w = f2_of(L::W(ip));
+        v[K] = pair_in(f[ip], f[ip + 1], w.hi, w.lo);
+      });
+    } else {
+      DF d[L::Q];
+      pull<L, P, DF>(fin, p, x, y, z, d);
+      d0 = d[0];
+      static_for<0, (L::Q - 1) / 2>([&](auto K) { v[K] = sum_diff(pack(d[2 * K + 1], d[2 * K + 2])); });
+    }
+    df2_store<L, FO>(d0, v, g, site, fout, p);
   }
 }
 
