@@ -821,15 +821,41 @@ int lbm_set_solid(lbm_ctx* c, const unsigned char* solid, const double* T_wall) 
   }
   if (!c->solid) {
     if (cudaMalloc(&c->solid, N) != cudaSuccess || cudaMalloc(&c->wall_th, N * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&c->wall_th_f, N * sizeof(float)) != cudaSuccess) {
+        cudaMalloc(&c->wall_th_f, N * sizeof(float)) != cudaSuccess || cudaMalloc(&c->site_class, N) != cudaSuccess) {
       cudaGetLastError();
       return fail(c, LBM_ENOMEM, "device allocation of the solid-site tables failed");
     }
-    c->bytes += N * (1 + sizeof(double) + sizeof(float));
+    c->bytes += N * (2 + sizeof(double) + sizeof(float));
   }
-  LBM_CUDA(c, cudaMemcpy(c->solid, s.data(), N, cudaMemcpyHostToDevice));
+  LBM_CUDA(c, cudaMemcpyAsync(c->solid, s.data(), N, cudaMemcpyHostToDevice, c->stream));
   LBM_CUDA(c, cudaMemcpy(c->wall_th, th.data(), N * sizeof(double), cudaMemcpyHostToDevice));
   LBM_CUDA(c, cudaMemcpy(c->wall_th_f, thf.data(), N * sizeof(float), cudaMemcpyHostToDevice));
+  // the fluid sites next to a solid one: counted, then listed
+  unsigned n_wall = 0;
+  LBM_CUDA(c, cudaMemsetAsync(c->ticket, 0, sizeof(unsigned), c->stream));
+  LBM_CUDA(c, c->ops->classify(c->solid, c->site_class, nullptr, c->ticket, 0, c->p, c->stream));
+  LBM_CUDA(c, cudaMemcpyAsync(&n_wall, c->ticket, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+  LBM_CUDA(c, cudaMemsetAsync(c->ticket, 0, sizeof(unsigned), c->stream));
+  LBM_CUDA(c, cudaStreamSynchronize(c->stream));
+  if (c->wall_sites) {  // set a second time before lbm_init
+    c->bytes -= sizeof(int) * (size_t)c->p.n_wall_sites;
+    cudaFree(c->wall_sites);
+    c->wall_sites = nullptr;
+  }
+  c->p.n_wall_sites = 0;
+  if (n_wall) {
+    if (cudaMalloc(&c->wall_sites, sizeof(int) * (size_t)n_wall) != cudaSuccess) {
+      cudaGetLastError();
+      return fail(c, LBM_ENOMEM, "device allocation of the wall-site list failed");
+    }
+    c->bytes += sizeof(int) * (size_t)n_wall;
+    LBM_CUDA(c, c->ops->classify(c->solid, c->site_class, c->wall_sites, c->ticket, 1, c->p, c->stream));
+    LBM_CUDA(c, cudaMemsetAsync(c->ticket, 0, sizeof(unsigned), c->stream));
+    LBM_CUDA(c, cudaStreamSynchronize(c->stream));
+  }
+  c->p.site_class = c->site_class;
+  c->p.wall_sites = c->wall_sites;
+  c->p.n_wall_sites = (int)n_wall;
   c->p.solid = c->solid;
   c->p.wall_th = c->wall_th;
   c->p.wall_th_f = c->wall_th_f;
@@ -1222,6 +1248,8 @@ void lbm_destroy(lbm_ctx* c) {
   cudaFree(c->gtab);
   cudaFree(c->gtab_f);
   cudaFree(c->solid);
+  cudaFree(c->site_class);
+  cudaFree(c->wall_sites);
   cudaFree(c->wall_th);
   cudaFree(c->wall_th_f);
   cudaFree(c->part);

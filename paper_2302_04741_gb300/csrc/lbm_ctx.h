@@ -41,6 +41,8 @@ struct lbm_ctx {
   double* gtab = nullptr;      // force table / field
   float* gtab_f = nullptr;     // its float copy (float kernels)
   unsigned char* solid = nullptr;  // solid-site flags (lbm_set_solid), N bytes
+  unsigned char* site_class = nullptr;  // fluid / solid / fluid next to a solid, N bytes
+  int* wall_sites = nullptr;   // the sites of the last class
   double* wall_th = nullptr;   // wall temperature - 1 per site, N doubles
   float* wall_th_f = nullptr;  // its float copy
   double* part = nullptr;      // conservation partials (CONS_SLOT doubles per block)

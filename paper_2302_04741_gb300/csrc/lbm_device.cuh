@@ -54,6 +54,11 @@ struct StepParams {
   // wall temperature minus 1 per site (read at solid sites only); nullptr
   // when the grid has none
   const unsigned char* solid;
+  // 0: fluid, 1: solid, 2: fluid with a solid pull source; the sites of class 2 as
+  // a list (the step gives them blocks of their own)
+  const unsigned char* site_class;
+  const int* wall_sites;
+  int n_wall_sites;
   const double* wall_th;
   const float* wall_th_f;
   int l2_evict_first;  // 1: population loads are evict-first in L2 (see ld_pop_policy)

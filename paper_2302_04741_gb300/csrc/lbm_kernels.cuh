@@ -593,36 +593,82 @@ __device__ __forceinline__ int launch_line(int b, int n, bool walls, int reverse
   return b < 3 ? b : (b < 6 ? n - 6 + b : (reverse ? n + 2 - b : b - 3));
 }
 
-// SOLID: the grid has solid sites (they are skipped; their fluid neighbours
-// take the diffuse-wall pull).
+// Class of every site of a grid with solid sites, and the list of the fluid
+// sites next to one: pass 0 counts them, pass 1 writes the list.
+template <class L>
+__global__ void __launch_bounds__(256) k_classify(const unsigned char* __restrict__ solid, unsigned char* __restrict__ cls,
+                                                  int* __restrict__ list, unsigned* __restrict__ count, int pass,
+                                                  const StepParams p) {
+  const int site = blockIdx.x * 256 + threadIdx.x;
+  if (site >= p.N) return;
+  unsigned char c = solid[site] ? 1 : 0;
+  if (!c) {
+    const int x = site % p.nx, row = site / p.nx, y = row % p.ny, z = row / p.ny;
+    static_for<1, L::Q>([&](auto I) {
+      constexpr int i = I;
+      const int sx = wrap3(x - L::E(i, 0), p.nx), sy = wrap3(y - L::E(i, 1), p.ny);
+      const int sz = L::D == 3 ? wrap3(z - L::E(i, 2), p.nz) : 0;
+      if (solid[(sz * p.ny + sy) * p.nx + sx]) c = 2;
+    });
+  }
+  if (pass == 0) cls[site] = c;
+  if (c == 2) {
+    const unsigned k = atomicAdd(count, 1u);
+    if (pass == 1) list[k] = site;
+  }
+}
+
+// Lines (y rows in 2-D, z layers in 3-D) that the list of wall sites adds in front
+// of a step's grid of blocks of bx threads.
+template <int D>
+inline int wall_site_lines(const StepParams& p, int bx) {
+  const long long line = (long long)((p.nx + bx - 1) / bx) * (D == 2 ? 1 : p.ny) * bx;
+  return (int)((p.n_wall_sites + line - 1) / line);
+}
+
+// SOLID: the grid has solid sites.  Solid sites are skipped; fluid sites next to
+// one take the diffuse-wall pull, in blocks of their own (the first of the
+// launch): left among the others, a warp with one such site ran the wall's FP64
+// operations for all 37 directions, 470 beside the 440 of a plain site, and every
+// site read 37 flags.  256 x 256 cylinders, 20 steps and read-out 1.37 -> 1.03 ms.
 template <class L, int P, int FO, bool SOLID = false>
 __global__ void __launch_bounds__(256, min_blocks<L, P>())
     k_step(const typename Codec<P>::T* __restrict__ fin, typename Codec<P>::T* __restrict__ fout,
            const StepParams p) {
   using R = typename Codec<P>::R;
+  const int lines = SOLID ? (int)(L::D == 2 ? gridDim.y : gridDim.z) - p.na : 0;  // of wall sites (wall_site_lines)
+  if constexpr (SOLID) {
+    const int line = L::D == 2 ? blockIdx.y : blockIdx.z;
+    if (line < lines) {
+      const int blk = (L::D == 2 ? line : line * p.ny + (int)blockIdx.y) * gridDim.x + blockIdx.x;
+      const int k = blk * blockDim.x + threadIdx.x;
+      asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+      if (k >= p.n_wall_sites) return;
+      const int site = __ldg(p.wall_sites + k), x = site % p.nx, row = site / p.nx, y = row % p.ny, z = row / p.ny;
+      R g[3];
+      site_force_r<L::D, R>(p, x, y, z, site, g);
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      R d[L::Q];
+      pull_solid<L, P, R>(fin, p, x, y, z, site, d);
+      if constexpr (P == P_FP64) {
+        R d0, s[(L::Q - 1) / 2], a[(L::Q - 1) / 2];
+        pair_split_dev<L, R>(d, d0, s, a);
+        poly_store<L, FO>(d0, s, a, g, site, fout, p);
+      } else {
+        collide_store<L, P, FO>(d, g, site, fout, p);
+      }
+      return;
+    }
+  }
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= p.nx) return;
   const bool walls = p.wall != W_NONE;
-  const int y = L::D == 2 ? p.a0 + launch_line(blockIdx.y, p.na, walls, p.reverse)
+  const int y = L::D == 2 ? p.a0 + launch_line(blockIdx.y - lines, p.na, walls, p.reverse)
                           : (p.reverse ? p.ny - 1 - (int)blockIdx.y : (int)blockIdx.y);
-  const int z = L::D == 3 ? p.a0 + launch_line(blockIdx.z, p.na, walls, p.reverse) : 0;
+  const int z = L::D == 3 ? p.a0 + launch_line(blockIdx.z - lines, p.na, walls, p.reverse) : 0;
   const int site = (z * p.ny + y) * p.nx + x;
   if constexpr (SOLID) {
-    if (__ldg(p.solid + site)) return;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    R g[3];
-    site_force_r<L::D, R>(p, x, y, z, site, g);
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    R d[L::Q];
-    pull_solid<L, P, R>(fin, p, x, y, z, site, d);
-    if constexpr (P == P_FP64) {
-      R d0, s[(L::Q - 1) / 2], a[(L::Q - 1) / 2];
-      pair_split_dev<L, R>(d, d0, s, a);
-      poly_store<L, FO>(d0, s, a, g, site, fout, p);
-    } else {
-      collide_store<L, P, FO>(d, g, site, fout, p);
-    }
-    return;
+    if (__ldg(p.site_class + site)) return;
   }
   const int a = L::D == 2 ? y : z;
   const int nA = L::D == 2 ? p.ny : p.nz;
@@ -1121,8 +1167,9 @@ __global__ void __launch_bounds__(128) k_moments(const typename Codec<P>::T* __r
   const int z = D == 3 ? p.a0 + (int)blockIdx.z : 0;
   const int site = (z * p.ny + y) * p.nx + x;
   const size_t N = (size_t)p.N;
+  const int cls = SOLID ? p.site_class[site] : 0;
   if constexpr (SOLID) {
-    if (p.solid[site]) {  // solid sites report zeros
+    if (cls == 1) {  // solid sites report zeros
       if (rho) rho[site] = 0.0;
       if (T) T[site] = 0.0;
       for (int a = 0; a < D; ++a) {
@@ -1148,11 +1195,11 @@ __global__ void __launch_bounds__(128) k_moments(const typename Codec<P>::T* __r
     write_moments<L, DF>(h, g, site, N, force_order, p, rho, u, T, q);
   } else {
     double d0, s[(Q - 1) / 2], a[(Q - 1) / 2];
-    if constexpr (SOLID) {
+    if (SOLID && cls) {
       double d[Q];
       pull_solid<L, P, double>(fin, p, x, y, z, site, d);
       pair_split_dev<L, double>(d, d0, s, a);
-    } else if (!near) {
+    } else if (P == P_FP64 && !near) {
       double f[Q];
       if (interior) pull_interior<L, P, double, LD_HINT, IN_STORED>(fin + site, p, y, z, f);
       else pull_stored<L, P, double>(fin, p, x, y, z, f);
@@ -1351,7 +1398,8 @@ __global__ void __launch_bounds__(128, LBM_CONSERVED_BLOCKS) k_conserved(const t
     const int x = xt * 128 + threadIdx.x;
     if (x >= p.nx) continue;
     const int site = (z * p.ny + y) * p.nx + x;
-    if (p.solid && p.solid[site]) continue;
+    const int cls = p.solid ? p.site_class[site] : 0;
+    if (cls == 1) continue;
     const int a = D == 2 ? y : z;
     const int nA = D == 2 ? p.ny : p.nz;
     const int wx0 = xt * 128 + (threadIdx.x & ~31);
@@ -1360,21 +1408,21 @@ __global__ void __launch_bounds__(128, LBM_CONSERVED_BLOCKS) k_conserved(const t
     RawMoments<L, R> r;
     if constexpr (P == P_FP64) {  // pair sums and mirror groups: fewer FP64 operations
       R d0, s[(Q - 1) / 2], am[(Q - 1) / 2];
-      if (!p.solid && !near) {
+      if (!cls && !near) {
         R f[Q];
         if (interior) pull_interior<L, P, R, LD_HINT, IN_STORED>(fin + site, p, y, z, f);
         else pull_stored<L, P, R>(fin, p, x, y, z, f);
         pair_split<L, R>(f, d0, s, am);
       } else {
         R d[Q];
-        if (p.solid) pull_solid<L, P, R>(fin, p, x, y, z, site, d);
+        if (cls) pull_solid<L, P, R>(fin, p, x, y, z, site, d);
         else pull<L, P, R>(fin, p, x, y, z, d);
         pair_split_dev<L, R>(d, d0, s, am);
       }
       r = pair_moments<L, R>(d0, s, am);
     } else {
       R d[Q];
-      if (p.solid) pull_solid<L, P, R>(fin, p, x, y, z, site, d);
+      if (cls) pull_solid<L, P, R>(fin, p, x, y, z, site, d);
       else if (interior) pull_interior<L, P, R>(fin + site, p, y, z, d);
       else pull<L, P, R>(fin, p, x, y, z, d);
       r = raw_moments<L, R>(d);

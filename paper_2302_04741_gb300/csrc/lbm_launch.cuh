@@ -28,6 +28,9 @@ struct LatticeOps {
                             const StepParams& p, int nsm, cudaStream_t s);
   int nshell;
   const double* shell_w;
+  // classes of the sites of a grid with solid sites (k_classify)
+  cudaError_t (*classify)(const unsigned char* solid, unsigned char* cls, int* list, unsigned* count, int pass,
+                          const StepParams& p, cudaStream_t s);
   cudaError_t (*moments)(int P, const void* fin, double* rho, double* u, double* T, double* q,
                          int FO, const StepParams& p, cudaStream_t s);
   // ticket != nullptr: the last block also reduces into out (see k_conserved)
@@ -130,6 +133,7 @@ struct Ops {
     cfg.numAttrs = overlap ? 1 : 0;
     cudaError_t e = cudaSuccess;
     if (p.solid) {
+      (L::D == 2 ? cfg.gridDim.y : cfg.gridDim.z) += wall_site_lines<L::D>(p, bx);
 #define LBM_SOLID_CASE(PP, FF)                                                                 \
   case PP * 4 + FF:                                                                            \
     e = cudaLaunchKernelEx(&cfg, k_step<L, PP, FF, true>, (const T<PP>*)fin, (T<PP>*)fout, p); \
@@ -201,6 +205,12 @@ struct Ops {
     const long long most = 4LL * (nsm > 0 ? nsm : 1);
     const unsigned blocks = (unsigned)((sites + 255) / 256 < most ? (sites + 255) / 256 : most);
     k_init_scale<L><<<blocks, 256, 0, s>>>(rho, u, T_, maxbits, FO, p);
+    return cudaGetLastError();
+  }
+
+  static cudaError_t classify(const unsigned char* solid, unsigned char* cls, int* list, unsigned* count, int pass,
+                              const StepParams& p, cudaStream_t s) {
+    k_classify<L><<<(unsigned)(((long long)p.N + 255) / 256), 256, 0, s>>>(solid, cls, list, count, pass, p);
     return cudaGetLastError();
   }
 
@@ -410,7 +420,7 @@ struct Ops {
   }
 
   static LatticeOps table() {
-    return LatticeOps{L::Q, L::D, &step, &init, &init_scale, L::NSHELL, L::shell_w, &moments, &conserved, &conserved_final, &pulled, &state,
+    return LatticeOps{L::Q, L::D, &step, &init, &init_scale, L::NSHELL, L::shell_w, &classify, &moments, &conserved, &conserved_final, &pulled, &state,
                       &tma_smem, &tma_prepare, &step_tma, &async_occupancy, &step_async,
                       &batch_occupancy, &batch_step, &batch_staged_occupancy, &batch_step_staged,
                       &wave_occupancy, &step_wave};
