@@ -261,6 +261,16 @@ __device__ __forceinline__ T ld_pop_policy(const T* ptr, bool evict_first) {
   }
 }
 
+// The wait of a programmatic dependent launch for the step before.  Populations are
+// read through the pointer that it returns: a read-only load (__ldg) of the kernel's
+// own argument is not held back by the wait, "memory" or not.  Through the argument,
+// the first rows of a 2050 x 501 FP16 grid were read while the step before wrote them.
+template <class T>
+__device__ __forceinline__ const T* wait_previous(const T* f) {
+  asm volatile("griddepcontrol.wait;" : "+l"(f) : : "memory");
+  return f;
+}
+
 // ------------------------------------------------------- storage codecs
 // decode(stored, i) -> deviation d_i = f_i - w_i ; encode(d_i, i) -> stored
 template <int P> struct Codec;

@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(128, LBM_HALF2_BLOCKS)
   const int row = (z * p.ny + y) * p.nx;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (near_wall(p, a, D == 2 ? p.ny : p.nz)) {  // block-uniform: a row of the wall rules, site by site
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    fin = wait_previous(fin);
 #pragma unroll 1
     for (int k = k0; k < k1; ++k) {
       const int x = (2 * blockIdx.x + k) * bx + threadIdx.x;
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(128, LBM_HALF2_BLOCKS)
     site_force_r<D, float>(p, x + 1, y, z, row + x + 1, gb);
     for (int c = 0; c < 3; ++c) g[c] = make_float2(ga[c], gb[c]);
   }
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  fin = wait_previous(fin);
   // Byte offsets of x - 3 .. x + 4 in a row, wrapped: the address of a load is
   // then a block-uniform row pointer plus one of them.
   unsigned xs[8];

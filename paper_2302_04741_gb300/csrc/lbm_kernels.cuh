@@ -647,7 +647,7 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
       const int site = __ldg(p.wall_sites + k), x = site % p.nx, row = site / p.nx, y = row % p.ny, z = row / p.ny;
       R g[3];
       site_force_r<L::D, R>(p, x, y, z, site, g);
-      asm volatile("griddepcontrol.wait;" ::: "memory");
+      fin = wait_previous(fin);
       R d[L::Q];
       pull_solid<L, P, R>(fin, p, x, y, z, site, d);
       if constexpr (P == P_FP64) {
@@ -681,7 +681,7 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   R g[3];
   site_force_r<L::D, R>(p, x, y, z, site, g);
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  fin = wait_previous(fin);
   if constexpr (std::is_same<R, float>::value) {
     constexpr bool SC = scaled_step<P, FO>();
     R d[L::Q];

@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_split(const double* __re
   double g3[3];
   site_force<2>(p, x, y, 0, site, g3);
   const double g[2] = {g3[0], g3[1]};
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  fin = wait_previous(fin);
   // ---- pull: the members + and - of each slot
   const int side = y < 3 ? 0 : 1;
   const bool near = near_wall(p, y, nA);
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_sym(const double* __rest
   double g3[3];
   site_force<2>(p, x, y, 0, site, g3);
   const double g[2] = {role ? g3[1] : g3[0], role ? g3[0] : g3[1]};  // local
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  fin = wait_previous(fin);
   const int side = y < 3 ? 0 : 1;
   const bool near = near_wall(p, y, nA);
   // the weights that differ between the lanes
