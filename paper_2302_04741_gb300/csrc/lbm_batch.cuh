@@ -7,7 +7,7 @@
 // run of blockDim.x * SPT consecutive sites of one grid's flattened index
 // (x fastest), so grids whose rows are shorter than a block keep every
 // thread busy; prefix[g] is the first global tile of grid g (prefix[ngrids]
-// = all tiles).  CTAs (several waves of the resident capacity) stride over
+// = all tiles).  CTAs (several waves of the resident capacity) take runs of
 // the global tiles, so grids of any mix of sizes share one launch, and every
 // site goes through exactly the device code of k_step (bit-identical
 // results to stepping each grid alone).
@@ -32,7 +32,8 @@ static_assert(sizeof(BatchGrid) % 16 == 0, "BatchGrid is copied as int4");
 // this copy).
 constexpr int BATCH_STAGED = (int)(offsetof(BatchGrid, p) + offsetof(StepParams, fw) + 15) / 16 * 16;
 
-// header[0] = number of grids, header[1] = number of tiles
+// header[0] = number of grids, header[1] = number of tiles, header[2] = tiles
+// per CTA (enough that the launch covers them all)
 template <class L, int P, int FO, int SPT>
 __global__ void __launch_bounds__(256, min_blocks<L, P>())
     k_step_batch(const BatchGrid* __restrict__ grids, const int* __restrict__ prefix,
@@ -46,12 +47,25 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
   const int ngrids = __ldg(header), ntiles = __ldg(header + 1);
   const int bx = blockDim.x, TW = bx * SPT;
   int gcur = -1;
-  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    int lo = 0, hi = ngrids;  // prefix[lo] <= t < prefix[hi]
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (__ldg(prefix + mid) <= t) lo = mid;
-      else hi = mid;
+  // A CTA takes a run of consecutive tiles: they share the grid, its staged
+  // parameters and the search for it but at a grid's end.  Rows at a wall pull
+  // through a call: their code, inline, made the loop spill (132 B on D3Q39), but for
+  // D2Q37 in FP32 (8 B), whose wall rows it would only delay (cells with two walls
+  // 94.5 us a step, 98.0 with the call).  GB300, against tiles gridDim.x apart, us a
+  // step: 64 ragged D2Q37 grids FP32 273 -> 252, FP16 241 -> 213; 24 D3Q39 boxes FP32
+  // 341 -> 333, FP16 302 -> 284.  The bound is the traffic (92 % of the copy rate on
+  // the FP32 D2Q37 mix).
+  const int run = __ldg(header + 2);
+  int next = 0, lo = 0;  // first tile of the next grid; this grid
+  for (int t = blockIdx.x * run, t1 = min(t + run, ntiles); t < t1; ++t) {
+    if (t >= next) {  // block-uniform
+      int hi = ngrids;  // prefix[lo] <= t < prefix[hi]
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(prefix + mid) <= t) lo = mid;
+        else hi = mid;
+      }
+      next = __ldg(prefix + lo + 1);
     }
     if (lo != gcur) {  // block-uniform
       __syncthreads();
@@ -85,7 +99,13 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
       constexpr bool SC = scaled_step<P, FO>();
       R d[L::Q];
       if (interior) pull_interior<L, P, R, LD_RO, SC ? IN_SCALED : IN_DEV>(fin + site, p, y, z, d);
-      else pull<L, P, R, LD_RO, SC>(fin, p, x, y, z, d);
+      else if (!near_wall(p, L::D == 2 ? y : z, nA)) pull_stored<L, P, R, LD_RO, SC ? IN_SCALED : IN_DEV>(fin, p, x, y, z, d);
+      else if (L::D == 2 && P == P_FP32S) pull<L, P, R, LD_RO, SC>(fin, p, x, y, z, d);
+      else {
+        R w[L::Q];
+        pull_call<L, P, LD_RO, SC>(fin, p, x, y, z, w);
+        static_for<0, L::Q>([&](auto I) { d[I] = w[I]; });
+      }
       R g[3];
       site_force_r<L::D, R>(p, x, y, z, site, g);
       collide_store<L, P, FO, SC>(d, g, site, fout, p);

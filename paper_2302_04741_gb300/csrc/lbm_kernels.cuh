@@ -73,9 +73,9 @@ __device__ __forceinline__ typename Codec<P>::R pulled_value(typename Codec<P>::
   else return step_in<L, P, I, IN == IN_SCALED>(v, p);
 }
 
-// Pull of the stored values of site (x, y, z) of a row that no wall rule
-// touches, with the periodic wrap of every axis.
-template <class L, int P, class RR, int LD = LD_HINT>
+// Pull of site (x, y, z) of a row that no wall rule touches, with the periodic
+// wrap of every axis (IN: what is returned, by default the stored values).
+template <class L, int P, class RR, int LD = LD_HINT, int IN = IN_STORED>
 __device__ __forceinline__ void pull_stored(const typename Codec<P>::T* __restrict__ fin,
                                           const StepParams& p, int x, int y, int z, RR (&d)[L::Q]) {
   using C = Codec<P>;
@@ -93,7 +93,7 @@ __device__ __forceinline__ void pull_stored(const typename Codec<P>::T* __restri
     constexpr int i = I;
     constexpr int ex = L::E(i, 0), ey = L::E(i, 1), ez = L::E(i, 2);
     const int off = zs[ez + 3] + ys[ey + 3] + xs[ex + 3];
-    d[i] = pulled_value<L, P, i, IN_STORED>(ldpop<C, LD>(fin + i * N + off, p), p);
+    d[i] = RR(pulled_value<L, P, i, IN>(ldpop<C, LD>(fin + i * N + off, p), p));
   });
 }
 
@@ -195,6 +195,16 @@ __device__ __forceinline__ void pull(const typename Codec<P>::T* __restrict__ fi
   // a row next to a wall (block-uniform side)
   if (a < 3) pull_near<L, P, RR, LD, SC, 0>(fin, p, x, y, z, a, nA, xs, ys, zs, d);
   else pull_near<L, P, RR, LD, SC, 1>(fin, p, x, y, z, a, nA, xs, ys, zs, d);
+}
+
+// The same into memory, as a call: for a kernel whose registers the wall rows'
+// code would overflow.
+template <class L, int P, int LD, bool SC>
+__device__ __noinline__ void pull_call(const typename Codec<P>::T* __restrict__ fin, const StepParams& p, int x, int y,
+                                       int z, typename Codec<P>::R* out) {
+  typename Codec<P>::R d[L::Q];
+  pull<L, P, typename Codec<P>::R, LD, SC>(fin, p, x, y, z, d);
+  static_for<0, L::Q>([&](auto I) { out[I] = d[I]; });
 }
 
 // ------------------------------------------------------- solid sites
