@@ -247,24 +247,25 @@ __device__ __forceinline__ T ld_pop_policy(const T* ptr, bool evict_first) {
   asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(first));
   asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(normal));
   const unsigned long long pol = evict_first ? first : normal;
-  // volatile, like the read-only-path intrinsics: the load stays after the
-  // griddepcontrol.wait of a programmatic dependent launch
+  // volatile and not .nc: the load stays after wait_previous
   if constexpr (sizeof(T) == 4) {
     float v;
-    asm volatile("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(ptr), "l"(pol));
+    asm volatile("ld.global.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(ptr), "l"(pol));
     return v;
   } else {
     static_assert(sizeof(T) == 2, "16- or 32-bit populations");
     unsigned short v;
-    asm volatile("ld.global.nc.L2::cache_hint.b16 %0, [%1], %2;" : "=h"(v) : "l"(ptr), "l"(pol));
+    asm volatile("ld.global.L2::cache_hint.b16 %0, [%1], %2;" : "=h"(v) : "l"(ptr), "l"(pol));
     return __ushort_as_half(v);
   }
 }
 
 // The wait of a programmatic dependent launch for the step before.  Populations are
-// read through the pointer that it returns: a read-only load (__ldg) of the kernel's
-// own argument is not held back by the wait, "memory" or not.  Through the argument,
-// the first rows of a 2050 x 501 FP16 grid were read while the step before wrote them.
+// read through the pointer that it returns, with plain loads: ld.global.nc is for
+// data that nobody writes while the kernel lives, which begins before the wait, so
+// such a load may be moved ahead of it ("memory" or a pointer that comes out of the
+// asm hold back the front end only).  It was: the first rows of a periodic FP16 grid
+// read the last ones while the step before still wrote them.
 template <class T>
 __device__ __forceinline__ const T* wait_previous(const T* f) {
   asm volatile("griddepcontrol.wait;" : "+l"(f) : : "memory");
@@ -282,7 +283,7 @@ template <> struct Codec<P_FP64> {
   __device__ __forceinline__ static R decode(T v, const StepParams&) { return v - L::W(I); }
   template <class L, int I>
   __device__ __forceinline__ static T encode(R d, const StepParams&) { return d + L::W(I); }
-  __device__ __forceinline__ static T load(const T* ptr, const StepParams&) { return __ldg(ptr); }
+  __device__ __forceinline__ static T load(const T* ptr, const StepParams&) { return *ptr; }
   __device__ __forceinline__ static T load_cg(const T* p) { return __ldcg(p); }
 };
 
@@ -314,7 +315,7 @@ template <> struct Codec<P_FP64DF> {
     constexpr DF w = DF(L::W(I));
     return df_to_double(d + w);
   }
-  __device__ __forceinline__ static T load(const T* ptr, const StepParams&) { return __ldg(ptr); }
+  __device__ __forceinline__ static T load(const T* ptr, const StepParams&) { return *ptr; }
   __device__ __forceinline__ static T load_cg(const T* p) { return __ldcg(p); }
 };
 
@@ -404,14 +405,15 @@ inline void set_fp16_factors(StepParams& p) {
 
 // Load modes of a population pull: LD_HINT the codec's load (float codecs:
 // the L2 policy of StepParams::l2_evict_first), LD_RO the plain read-only
-// path (for kernels at their register cap: the policy costs two registers),
-// LD_CG from L2 only (for a kernel that reads what other blocks of the same
+// path (for kernels at their register cap: the policy costs two registers; not after
+// wait_previous), LD_PLAIN the same as a plain load, LD_CG from L2 only (for a kernel that reads what other blocks of the same
 // launch wrote: the read-only and L1 paths may hold stale lines).
-enum { LD_HINT = 0, LD_RO = 1, LD_CG = 2 };
+enum { LD_HINT = 0, LD_RO = 1, LD_CG = 2, LD_PLAIN = 3 };
 template <class C, int LD>
 __device__ __forceinline__ typename C::T ldpop(const typename C::T* ptr, const StepParams& p) {
   if constexpr (LD == LD_CG) return C::load_cg(ptr);
   else if constexpr (LD == LD_RO) return __ldg(ptr);
+  else if constexpr (LD == LD_PLAIN) return *ptr;
   else return C::load(ptr, p);
 }
 

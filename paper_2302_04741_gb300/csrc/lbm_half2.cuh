@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(128, LBM_HALF2_BLOCKS)
       if (x >= p.nx) break;
       float g[3], d[Q];
       site_force_r<D, float>(p, x, y, z, row + x, g);
-      pull<L, P_FP16S, float, LD_RO, true>(fin, p, x, y, z, d);
+      pull<L, P_FP16S, float, LD_PLAIN, true>(fin, p, x, y, z, d);
       collide_store<L, P_FP16S, FO, true>(d, g, row + x, fout, p);
     }
     return;
@@ -267,10 +267,10 @@ __global__ void __launch_bounds__(128, LBM_HALF2_BLOCKS)
     constexpr int i = I, ex = L::E(i, 0), k = 3 - ex;
     const char* src = reinterpret_cast<const char*>(fin + (i * N + (size_t)(zs[L::E(i, 2) + 3] + ys[L::E(i, 1) + 3])));
     if constexpr (ex % 2 == 0) {  // x and nx even: the two sources are one aligned word
-      h[i] = __ldg(reinterpret_cast<const unsigned*>(src + xs[k]));
+      h[i] = *reinterpret_cast<const unsigned*>(src + xs[k]);
     } else {
-      const unsigned lo = __ldg(reinterpret_cast<const unsigned short*>(src + xs[k]));
-      const unsigned hi = __ldg(reinterpret_cast<const unsigned short*>(src + xs[k + 1]));
+      const unsigned lo = *reinterpret_cast<const unsigned short*>(src + xs[k]);
+      const unsigned hi = *reinterpret_cast<const unsigned short*>(src + xs[k + 1]);
       h[i] = lo | hi << 16;
     }
   });

@@ -147,8 +147,8 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_split(const double* __re
         xm = x;
       }
     }
-    fp[r] = __ldg(fin + (jp * N + (size_t)(yp * nx + xp)));
-    fm[r] = __ldg(fin + (jm * N + (size_t)(ym * nx + xm)));
+    fp[r] = fin[(jp * N + (size_t)(yp * nx + xp))];
+    fm[r] = fin[(jm * N + (size_t)(ym * nx + xm))];
   }
   // what leaves the column through a thermal wall, loaded with the pull: one
   // latency for both (as loops of their own they took 3 us a step)
@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_split(const double* __re
       const int t = lane + r * G;
       if (t < SPLIT_LEAVES) {
         const int j = leave_j[r], row = side == 0 ? leave_r[r] : nA - 1 - leave_r[r];
-        leave[r] = __ldg(fin + ((side == 0 ? j : ((j & 1) ? j + 1 : j - 1)) * N + (size_t)(row * nx + x)));
+        leave[r] = fin[((side == 0 ? j : ((j & 1) ? j + 1 : j - 1)) * N + (size_t)(row * nx + x))];
       }
     }
   }
@@ -335,10 +335,10 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_sym(const double* __rest
         xm = x;
       }
     }
-    fp[k] = __ldg(fin + (jp * N + (size_t)(yp * nx + xp)));
-    fm[k] = __ldg(fin + (jm * N + (size_t)(ym * nx + xm)));
+    fp[k] = fin[(jp * N + (size_t)(yp * nx + xp))];
+    fm[k] = fin[(jm * N + (size_t)(ym * nx + xm))];
   });
-  const double f0 = __ldg(fin + site);
+  const double f0 = fin[site];
   const bool thermal = p.wall == W_THERMAL && near;
   const bool any_thermal = __any_sync(ALL, thermal);  // warp-uniform
   double leave[SPLIT_LEAVES / 2] = {};  // of the column through a thermal wall: every other one
@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_sym(const double* __rest
       constexpr int j0 = t.leave_j[2 * T], j1 = t.leave_j[2 * T + 1], r0 = t.leave_r[2 * T], r1 = t.leave_r[2 * T + 1];
       const int j = role ? j1 : j0, r = role ? r1 : r0;
       const int js = side == 0 ? j : (j & 1 ? j + 1 : j - 1), row = side == 0 ? r : nA - 1 - r;
-      leave[T] = __ldg(fin + (js * N + (size_t)(row * nx + x)));
+      leave[T] = fin[(js * N + (size_t)(row * nx + x))];
     });
   }
   double rm1 = 0.0;
