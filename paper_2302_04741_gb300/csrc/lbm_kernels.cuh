@@ -104,12 +104,12 @@ __device__ __forceinline__ bool near_wall(const StepParams& p, int a, int nA) {
 
 // sum + the deviation of a stored value of wall row ROW, in the sum of a thermal
 // wall.  FP16 storage: the decode's product is fused into the sum, but for the
-// row-2 population of D3Q39 (0, 0, +-3), which is rounded first (written out, so
-// that every kernel forms the same wall density).
+// row-2 population along the wall's normal, (0, +-3) or (0, 0, +-3), which is rounded
+// first (written out, so that every kernel forms the same wall density).
 template <class L, int P, int J, int ROW, class RR>
 __device__ __forceinline__ RR add_deviation(RR sum, typename Codec<P>::T v, const StepParams& p) {
   if constexpr (P == P_FP16S && std::is_same<RR, float>::value) {
-    if constexpr (L::D == 3 && ROW == 2) return __fadd_rn(sum, __fmul_rn(__half2float(v), p.h_dec[J]));
+    if constexpr (ROW == 2 && L::E(J, 0) == 0 && (L::D == 2 || L::E(J, 1) == 0)) return __fadd_rn(sum, __fmul_rn(__half2float(v), p.h_dec[J]));
     else return fmaf(__half2float(v), p.h_dec[J], sum);
   } else {
     return sum + RR(Codec<P>::template decode<L, J>(v, p));
