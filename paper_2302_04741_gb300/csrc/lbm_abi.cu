@@ -830,7 +830,7 @@ int lbm_set_solid(lbm_ctx* c, const unsigned char* solid, const double* T_wall) 
   LBM_CUDA(c, cudaMemcpyAsync(c->solid, s.data(), N, cudaMemcpyHostToDevice, c->stream));
   LBM_CUDA(c, cudaMemcpy(c->wall_th, th.data(), N * sizeof(double), cudaMemcpyHostToDevice));
   LBM_CUDA(c, cudaMemcpy(c->wall_th_f, thf.data(), N * sizeof(float), cudaMemcpyHostToDevice));
-  // the fluid sites next to a solid one: counted, then listed
+  // the fluid sites next to a solid one: counted, then listed (wall_list)
   unsigned n_wall = 0;
   LBM_CUDA(c, cudaMemsetAsync(c->ticket, 0, sizeof(unsigned), c->stream));
   LBM_CUDA(c, c->ops->classify(c->solid, c->site_class, nullptr, c->ticket, 0, c->p, c->stream));
@@ -843,6 +843,7 @@ int lbm_set_solid(lbm_ctx* c, const unsigned char* solid, const double* T_wall) 
     c->wall_sites = nullptr;
   }
   c->p.n_wall_sites = 0;
+  if (!lbm::wall_list(c->opt.precision, c->N)) n_wall = 0;
   if (n_wall) {
     if (cudaMalloc(&c->wall_sites, sizeof(int) * (size_t)n_wall) != cudaSuccess) {
       cudaGetLastError();

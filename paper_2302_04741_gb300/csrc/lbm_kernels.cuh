@@ -628,6 +628,18 @@ __global__ void __launch_bounds__(256) k_classify(const unsigned char* __restric
   }
 }
 
+// Whether a grid keeps the list of its wall sites (SOLID_LIST): the FP64 step once it
+// fills the chip.  Below, a step lasts as long as one warp's pull, and a warp of
+// listed sites, whose missing slots differ, runs every slot's wall branch.  GB300,
+// cylinders in FP64, us for 40 steps alone / per grid with three at once, list then in
+// place: 160 x 160 2809 / 1220, 2303 / 1145; 176 x 176 2830 / 1278, 2766 / 1335;
+// 224 x 224 2882 / 1562, 2579 / 1912.  In FP32 the branches are cheap and the list
+// never paid (192 x 192: 18.9 us a step, 11.6 in place).
+#ifndef LBM_WALL_LIST_MIN_SITES
+#define LBM_WALL_LIST_MIN_SITES 28672
+#endif
+inline bool wall_list(int precision, long long sites) { return precision == P_FP64 && sites >= LBM_WALL_LIST_MIN_SITES; }
+
 // Lines (y rows in 2-D, z layers in 3-D) that the list of wall sites adds in front
 // of a step's grid of blocks of bx threads.
 template <int D>
@@ -636,18 +648,22 @@ inline int wall_site_lines(const StepParams& p, int bx) {
   return (int)((p.n_wall_sites + line - 1) / line);
 }
 
-// SOLID: the grid has solid sites.  Solid sites are skipped; fluid sites next to
-// one take the diffuse-wall pull, in blocks of their own (the first of the
-// launch): left among the others, a warp with one such site ran the wall's FP64
-// operations for all 37 directions, 470 beside the 440 of a plain site, and every
-// site read 37 flags.  256 x 256 cylinders, 20 steps and read-out 1.37 -> 1.03 ms.
-template <class L, int P, int FO, bool SOLID = false>
+// SOLID: the grid has solid sites.  They are skipped; fluid sites next to one take
+// the diffuse-wall pull.
+//   SOLID_LIST (wall_list): those sites in blocks of their own, the first of the
+//   launch.  Left among the others, a warp with one such site ran the wall's FP64
+//   operations for all 37 directions, 470 beside the 440 of a plain site, and every
+//   site read 37 flags.  256 x 256 cylinders FP64, 20 steps and read-out 1.37 -> 1.03 ms.
+//   SOLID_PLACE: among the others, in FP64 only in the warps that have such a site
+//   (146 x 146 cylinders, 40 steps and read-out 2.32 -> 1.87 ms, every site before).
+enum { SOLID_NONE = 0, SOLID_PLACE = 1, SOLID_LIST = 2 };
+template <class L, int P, int FO, int SOLID = SOLID_NONE>
 __global__ void __launch_bounds__(256, min_blocks<L, P>())
     k_step(const typename Codec<P>::T* __restrict__ fin, typename Codec<P>::T* __restrict__ fout,
            const StepParams p) {
   using R = typename Codec<P>::R;
-  const int lines = SOLID ? (int)(L::D == 2 ? gridDim.y : gridDim.z) - p.na : 0;  // of wall sites (wall_site_lines)
-  if constexpr (SOLID) {
+  const int lines = SOLID == SOLID_LIST ? (int)(L::D == 2 ? gridDim.y : gridDim.z) - p.na : 0;  // of wall sites (wall_site_lines)
+  if constexpr (SOLID == SOLID_LIST) {
     const int line = L::D == 2 ? blockIdx.y : blockIdx.z;
     if (line < lines) {
       const int blk = (L::D == 2 ? line : line * p.ny + (int)blockIdx.y) * gridDim.x + blockIdx.x;
@@ -677,8 +693,14 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
                           : (p.reverse ? p.ny - 1 - (int)blockIdx.y : (int)blockIdx.y);
   const int z = L::D == 3 ? p.a0 + launch_line(blockIdx.z - lines, p.na, walls, p.reverse) : 0;
   const int site = (z * p.ny + y) * p.nx + x;
-  if constexpr (SOLID) {
+  if constexpr (SOLID == SOLID_LIST) {
     if (__ldg(p.site_class + site)) return;
+  }
+  bool at_solid = false;  // a lane of this warp is next to a solid site
+  if constexpr (SOLID == SOLID_PLACE) {
+    const int cls = __ldg(p.site_class + site);
+    at_solid = P != P_FP64 || __any_sync(__activemask(), cls == 2);
+    if (cls == 1) return;
   }
   const int a = L::D == 2 ? y : z;
   const int nA = L::D == 2 ? p.ny : p.nz;
@@ -695,12 +717,17 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
   if constexpr (std::is_same<R, float>::value) {
     constexpr bool SC = scaled_step<P, FO>();
     R d[L::Q];
-    if (interior) pull_interior<L, P, R, LD_HINT, SC ? IN_SCALED : IN_DEV>(fin + site, p, y, z, d);
+    if (SOLID == SOLID_PLACE && at_solid) pull_solid<L, P, R>(fin, p, x, y, z, site, d);
+    else if (interior) pull_interior<L, P, R, LD_HINT, SC ? IN_SCALED : IN_DEV>(fin + site, p, y, z, d);
     else pull<L, P, R, LD_HINT, SC>(fin, p, x, y, z, d);
     collide_store<L, P, FO, SC>(d, g, site, fout, p);
   } else if constexpr (P == P_FP64) {
     R d0, s[(L::Q - 1) / 2], am[(L::Q - 1) / 2];
-    if (!near) {
+    if (SOLID == SOLID_PLACE && at_solid) {
+      R d[L::Q];
+      pull_solid<L, P, R>(fin, p, x, y, z, site, d);
+      pair_split_dev<L, R>(d, d0, s, am);
+    } else if (!near) {
       R f[L::Q];
       if (interior) pull_interior<L, P, R, LD_HINT, IN_STORED>(fin + site, p, y, z, f);
       else pull_stored<L, P, R>(fin, p, x, y, z, f);
@@ -1205,7 +1232,7 @@ __global__ void __launch_bounds__(128) k_moments(const typename Codec<P>::T* __r
     write_moments<L, DF>(h, g, site, N, force_order, p, rho, u, T, q);
   } else {
     double d0, s[(Q - 1) / 2], a[(Q - 1) / 2];
-    if (SOLID && cls) {
+    if (SOLID && __any_sync(__activemask(), cls)) {  // the warp as one: its lanes would take both pulls in turn
       double d[Q];
       pull_solid<L, P, double>(fin, p, x, y, z, site, d);
       pair_split_dev<L, double>(d, d0, s, a);

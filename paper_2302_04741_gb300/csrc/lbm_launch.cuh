@@ -133,16 +133,21 @@ struct Ops {
     cfg.numAttrs = overlap ? 1 : 0;
     cudaError_t e = cudaSuccess;
     if (p.solid) {
-      (L::D == 2 ? cfg.gridDim.y : cfg.gridDim.z) += wall_site_lines<L::D>(p, bx);
-#define LBM_SOLID_CASE(PP, FF)                                                                 \
-  case PP * 4 + FF:                                                                            \
-    e = cudaLaunchKernelEx(&cfg, k_step<L, PP, FF, true>, (const T<PP>*)fin, (T<PP>*)fout, p); \
+      if (p.wall_sites) (L::D == 2 ? cfg.gridDim.y : cfg.gridDim.z) += wall_site_lines<L::D>(p, bx);
+#define LBM_SOLID_CASE(PP, FF, SS)                                                           \
+  case (SS * 2 + PP) * 4 + FF:                                                               \
+    e = cudaLaunchKernelEx(&cfg, k_step<L, PP, FF, SS>, (const T<PP>*)fin, (T<PP>*)fout, p); \
     break;
-      switch (P * 4 + FO) {
-        LBM_SOLID_CASE(0, 0) LBM_SOLID_CASE(0, 1) LBM_SOLID_CASE(0, 2) LBM_SOLID_CASE(0, 3)
-        LBM_SOLID_CASE(1, 0) LBM_SOLID_CASE(1, 1) LBM_SOLID_CASE(1, 2) LBM_SOLID_CASE(1, 3)
+#define LBM_SOLID_CASES(PP, SS) \
+  LBM_SOLID_CASE(PP, 0, SS) LBM_SOLID_CASE(PP, 1, SS) LBM_SOLID_CASE(PP, 2, SS) LBM_SOLID_CASE(PP, 3, SS)
+      if (P != P_FP64 && P != P_FP32S) return cudaErrorInvalidValue;
+      switch (((p.wall_sites ? SOLID_LIST : SOLID_PLACE) * 2 + P) * 4 + FO) {
+        LBM_SOLID_CASES(P_FP64, SOLID_PLACE)
+        LBM_SOLID_CASES(P_FP32S, SOLID_PLACE)
+        LBM_SOLID_CASES(P_FP64, SOLID_LIST)
         default: return cudaErrorInvalidValue;
       }
+#undef LBM_SOLID_CASES
 #undef LBM_SOLID_CASE
       return e != cudaSuccess ? e : cudaGetLastError();
     }
