@@ -191,27 +191,24 @@ __device__ __forceinline__ void poly_coef2(const SiteState<DF>& m, PolyCoef2<DF>
   const DF2 XX = U * U;
   const DF xy = m.U[0] * m.U[1];
   const DF hu2 = half_of(m.u2);
-  const DF h = DF(0.5) - hmac(hu2, m.Th);
-  const DF2 AX = both(m.T) + XX;
+  const DF b0 = DF(1) - kmac<2>(m.Th, hu2);
+  const DF2 AX = both(m.T) + XX, HAX = DF2{__fmul2_rn(f2(0.5f, 0.5f), AX.hi), __fmul2_rn(f2(0.5f, 0.5f), AX.lo)};
   const DF T3 = kscale<3>(m.T), th2 = half_of(m.Th);
   const DF2 T3X = both(T3) + XX;
   const DF a00 = fma(hmac(half_of(hu2), m.Th), m.u2, fma(m.Th, m.Th, -(hu2 + m.Th)));
-  k.E00 = fma(m.rom, a00, m.om * m.drho);
-  DF2 E2 = both(m.rom) * fma(both(h), AX, -(both(th2) * XX));
-  k.E11 = kscale<2>(m.rom) * (h - th2) * xy;
+  k.E00 = fma(m.rom, a00, FO >= 1 ? fma(m.om, m.drho, -m.rkgu) : m.om * m.drho);
+  DF2 E2 = both(m.rom) * fma(both(b0), HAX, -(both(th2) * XX));
+  k.E11 = m.rom * (b0 - m.Th) * xy;
   const DF q = m.rom * DF(1.0 / 24.0);
   const DF2 E4 = both(q) * fma(XX, kmac<2>(both(T3), XX), both(T3 * m.T));
-  const DF2 E3 = both(kscale<4>(q) * xy) * T3X;
-  k.E22 = half_of(half_of(m.rom)) * px(AX) * py(AX);
-  const DF b0 = DF(1) - kmac<2>(m.Th, hu2);
+  k.E22 = m.rom * px(HAX) * py(HAX);
   const DF2 R = both(m.rom) * U;
   DF2 O3 = cmul2(1.0 / 6.0, 1.0 / 6.0, R) * T3X;
+  const DF2 E3 = O3 * DF2{f2(U.hi.y, U.hi.x), f2(U.lo.y, U.lo.x)};
   if constexpr (FO >= 1) {
-    k.E00 = k.E00 - m.rkgu;
     E2 = fma(S, U, E2);
     k.E11 = fma(m.S[0], m.U[1], fma(m.S[1], m.U[0], k.E11));
   }
-  const DF2 HAX = DF2{__fmul2_rn(f2(0.5f, 0.5f), AX.hi), __fmul2_rn(f2(0.5f, 0.5f), AX.lo)};
   DF2 O1, O2;
   if constexpr (FO >= 2) {
     const DF2 P = R + S;

@@ -462,22 +462,22 @@ __device__ __forceinline__ void site_coefficients(const RawMoments<L, R>& r, con
   constexpr int D = L::D;
   m.drho = r.drho;
   m.rho = R(1) + r.drho;
-  const R irho = R(1) / m.rho;
+  const R irho = R(1) / m.rho, cirho = mul_c<L, R>(irho);
   R u[3] = {R(0), R(0), R(0)};
-  R ut2 = R(0), g2 = R(0), gu = R(0);
+  R gu = R(0);
   m.u2 = R(0);
   for (int c = 0; c < D; ++c) {
-    const R ut = mul_c<L, R>(r.j[c] * irho);
-    u[c] = hmac(g[c], ut);
-    ut2 = c == 0 ? ut * ut : fma(ut, ut, ut2);
-    g2 = c == 0 ? g[c] * g[c] : fma(g[c], g[c], g2);
+    u[c] = hmac(g[c], r.j[c] * cirho);
     m.u2 = c == 0 ? u[c] * u[c] : fma(u[c], u[c], m.u2);
     gu = c == 0 ? g[c] * u[c] : fma(g[c], u[c], gu);
   }
-  m.Th = fma(fma(mul_c2<L, R>(r.k2) - kscale<D>(r.drho), irho, -ut2), R(1.0 / D), g2 * R(0.25 / D));
+  // D Th = k2 / rho - |u - g/2|^2 + g^2/4
+  const R DTh = fma(cmac(L::c2, r.k2, -kscale<D>(r.drho)), irho, gu - m.u2);
+  if constexpr (D == 2) m.Th = half_of(DTh);
+  else m.Th = DTh * R(1.0 / D);
   m.om = site_omega<R>(p, m.rho, R(1) + m.Th);
   m.rom = m.rho * m.om;
-  const R rk = m.rho - half_of(m.rom);
+  const R rk = hmac(-m.rom, m.rho);
   m.rkgu = FO >= 1 ? rk * gu : R(0);
   m.T = mul_c2<L, R>(m.Th);
   const R crk = mul_c<L, R>(rk);

@@ -204,15 +204,15 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_split(const double* __re
   m.drho = m0;
   m.rho = 1.0 + m0;
   const double irho = 1.0 / m.rho;
-  const double utx = L::c * (jx * irho), uty = L::c * (jy * irho);
-  const double ux = fma(0.5, g[0], utx), uy = fma(0.5, g[1], uty);
-  const double ut2 = fma(uty, uty, utx * utx), g2 = fma(g[1], g[1], g[0] * g[0]);
+  const double cirho = L::c * irho;
+  const double ux = fma(0.5, g[0], jx * cirho), uy = fma(0.5, g[1], jy * cirho);
+  const double gu = fma(g[1], uy, g[0] * ux);
   m.u2 = fma(uy, uy, ux * ux);
-  m.Th = fma(fma(fma(L::c2, k2, -2.0 * m0), irho, -ut2), 0.5, 0.125 * g2);
+  m.Th = 0.5 * fma(fma(L::c2, k2, -2.0 * m0), irho, gu - m.u2);
   m.om = site_omega<double>(p, m.rho, 1.0 + m.Th);
   m.rom = m.rho * m.om;
   const double rk = fma(-0.5, m.rom, m.rho);
-  m.rkgu = FO >= 1 ? rk * fma(g[1], uy, g[0] * ux) : 0.0;
+  m.rkgu = FO >= 1 ? rk * gu : 0.0;
   m.T = L::c2 * m.Th;
   const double crk = L::c * rk;
   m.U[0] = L::c * ux;
@@ -409,15 +409,15 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_sym(const double* __rest
   jy += jxo;
   // ---- mid-point state (local frame)
   const double rho = 1.0 + m0, irho = 1.0 / rho;
-  const double utx = L::c * (jx * irho), uty = L::c * (jy * irho);
-  const double ux = fma(0.5, g[0], utx), uy = fma(0.5, g[1], uty);
-  const double ut2 = fma(uty, uty, utx * utx), g2 = fma(g[1], g[1], g[0] * g[0]);
+  const double cirho = L::c * irho;
+  const double ux = fma(0.5, g[0], jx * cirho), uy = fma(0.5, g[1], jy * cirho);
+  const double gu = fma(g[1], uy, g[0] * ux);
   const double u2 = fma(uy, uy, ux * ux);
-  const double Th = fma(fma(fma(L::c2, k2, -2.0 * m0), irho, -ut2), 0.5, 0.125 * g2);
+  const double Th = 0.5 * fma(fma(L::c2, k2, -2.0 * m0), irho, gu - u2);
   const double om = site_omega<double>(p, rho, 1.0 + Th);
   const double rom = rho * om;
   const double rk = fma(-0.5, rom, rho);
-  const double rkgu = FO >= 1 ? rk * fma(g[1], uy, g[0] * ux) : 0.0;
+  const double rkgu = FO >= 1 ? rk * gu : 0.0;
   const double T = L::c2 * Th;
   const double crk = L::c * rk;
   const double X = L::c * ux, Y = L::c * uy, Sx = crk * g[0], Sy = crk * g[1];
@@ -425,23 +425,19 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_sym(const double* __rest
   PolyCoef2<double> c;
   {
     const double xx = X * X, xy = X * Y;
-    const double hu2 = 0.5 * u2;
-    const double h = 0.5 - fma(0.5, hu2, Th);
-    const double ax = T + xx, T3 = 3.0 * T, T3x = T3 + xx, th2 = 0.5 * Th;
-    const double a00 = fma(fma(0.25, hu2, Th), u2, fma(Th, Th, -(hu2 + Th)));
-    c.E00 = fma(rom, a00, om * m0);
-    const double qr = rom * (1.0 / 24.0), q4xy = 4.0 * qr * xy;
-    const double b0 = 1.0 - fma(2.0, Th, hu2);
+    const double b0 = fma(-0.5, u2, fma(-2.0, Th, 1.0));
+    const double hax = 0.5 * (T + xx), T3 = 3.0 * T, T3x = T3 + xx, th2 = 0.5 * Th;
+    const double a00 = fma(fma(0.125, u2, Th), u2, fma(Th, Th, fma(-0.5, u2, -Th)));
+    c.E00 = fma(rom, a00, FO >= 1 ? fma(om, m0, -rkgu) : om * m0);
+    const double qr = rom * (1.0 / 24.0);
     const double rx = rom * X;
-    c.E20 = rom * fma(h, ax, -(th2 * xx));
-    c.E11 = 2.0 * rom * (h - th2) * xy;
+    c.E20 = rom * fma(b0, hax, -(th2 * xx));
+    c.E11 = rom * (b0 - Th) * xy;
     c.E40 = qr * fma(xx, fma(2.0, T3, xx), T3 * T);
-    c.E31 = q4xy * T3x;
-    c.E22 = 0.25 * rom * ax * other(ax);
+    c.E22 = rom * hax * other(hax);
     c.O30 = (1.0 / 6.0) * rx * T3x;
-    const double hax = 0.5 * ax;
+    c.E31 = c.O30 * Y;
     if constexpr (FO >= 1) {
-      c.E00 -= rkgu;
       c.E20 = fma(Sx, X, c.E20);
       c.E11 = fma(Sx, Y, fma(Sy, X, c.E11));
     }
