@@ -568,8 +568,8 @@ __device__ __forceinline__ void df2_store(DF d0, const DF2 (&v)[(L::Q - 1) / 2],
 #ifndef LBM_FLOAT_D3Q39_BLOCKS
 #define LBM_FLOAT_D3Q39_BLOCKS 3
 #endif
-// LBM_DF_BLOCKS: the same for the float-float FP64 step (2: 128 registers, no
-// spill on D2Q37, ~250 B on D3Q39).
+// LBM_DF_BLOCKS: the same for the float-float FP64 step (2: 128 registers,
+// about 160 B of spill on D2Q37 and 190 B on D3Q39, mostly around its two calls).
 #ifndef LBM_DF_BLOCKS
 #define LBM_DF_BLOCKS 2
 #endif

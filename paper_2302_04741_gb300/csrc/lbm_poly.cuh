@@ -21,8 +21,8 @@
 //
 // Measured on GB300 (ten steps of 1024 x 512 D2Q37 sites and their read-out,
 // against the same body evaluated pair by pair in t = xi.u): IEEE double 6.46 ->
-// 4.73 ms, float-float 2.51 -> 1.70 ms (with df_split free of conversions);
-// D3Q39, 61 x 47 x 53 in double, 20 steps: 3.60 -> 2.88 ms.
+// 4.46 ms; float-float 2.51 -> 1.70 ms (with df_split free of conversions), 1.33 ms
+// in packed FP32 (lbm_df2.cuh); D3Q39, 61 x 47 x 53 in double, 20 steps: 3.60 -> 2.72 ms.
 #pragma once
 
 #include "lbm_device.cuh"
