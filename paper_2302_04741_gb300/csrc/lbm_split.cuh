@@ -204,11 +204,14 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_split(const double* __re
   m.drho = m0;
   m.rho = 1.0 + m0;
   const double irho = 1.0 / m.rho;
-  const double cirho = L::c * irho;
-  const double ux = fma(0.5, g[0], jx * cirho), uy = fma(0.5, g[1], jy * cirho);
+  // The temperature from j / rho and g: from u and g.u (site_coefficients) the errors of a
+  // steady 150-row channel rose by a quarter (T) and an eighth (q) for 1 % of the time.
+  const double utx = L::c * (jx * irho), uty = L::c * (jy * irho);
+  const double ux = fma(0.5, g[0], utx), uy = fma(0.5, g[1], uty);
+  const double ut2 = fma(uty, uty, utx * utx), g2 = fma(g[1], g[1], g[0] * g[0]);
   const double gu = fma(g[1], uy, g[0] * ux);
   m.u2 = fma(uy, uy, ux * ux);
-  m.Th = 0.5 * fma(fma(L::c2, k2, -2.0 * m0), irho, gu - m.u2);
+  m.Th = fma(fma(fma(L::c2, k2, -2.0 * m0), irho, -ut2), 0.5, 0.125 * g2);
   m.om = site_omega<double>(p, m.rho, 1.0 + m.Th);
   m.rom = m.rho * m.om;
   const double rk = fma(-0.5, m.rom, m.rho);
