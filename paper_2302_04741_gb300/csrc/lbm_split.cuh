@@ -28,11 +28,11 @@
 
 namespace lbm {
 
-// Doubles of a pair slot: e, the products of its components, the weight, |e|^2,
-// and the factor m of the pair sum in the density (1; 1/2 for the rest
+// Doubles of a pair slot: e, the products of its components, the weight, that of the
+// collision (collision_w), |e|^2, and the factor m of the pair sum in the density (1; 1/2 for the rest
 // particle, the last slot, which enters with both members equal).
 struct SplitSlot {
-  double x, y, xx, xy, yy, w, e2, m;
+  double x, y, xx, xy, yy, w, wg, e2, m;
 };
 constexpr int SPLIT_SLOTS = 19;
 constexpr int SPLIT_LEAVES = 26;
@@ -49,7 +49,7 @@ __host__ __device__ constexpr SplitTable make_split_table() {
   for (int k = 0; k < SPLIT_SLOTS; ++k) {
     const int i = k < SPLIT_SLOTS - 1 ? 2 * k + 1 : 0;
     const double x = L::e[i][0], y = L::e[i][1];
-    t.s[k] = SplitSlot{x, y, x * x, x * y, y * y, L::w[i], x * x + y * y, i ? 1.0 : 0.5};
+    t.s[k] = SplitSlot{x, y, x * x, x * y, y * y, L::w[i], collision_w<L>(i), x * x + y * y, i ? 1.0 : 0.5};
   }
   int n = 0;
   for (int j = 0; j < L::Q; ++j)
@@ -204,10 +204,10 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_split(const double* __re
   m.drho = m0;
   m.rho = 1.0 + m0;
   const double irho = 1.0 / m.rho;
-  // The temperature from j / rho and g: from u and g.u (site_coefficients) the errors of a
-  // steady 150-row channel rose by a quarter (T) and an eighth (q) for 1 % of the time.
-  const double utx = L::c * (jx * irho), uty = L::c * (jy * irho);
-  const double ux = fma(0.5, g[0], utx), uy = fma(0.5, g[1], uty);
+  // u and the temperature as in site_coefficients
+  const double cirho = L::c * irho, hgx = 0.5 * g[0], hgy = 0.5 * g[1];
+  const double ux = fma(jx, cirho, hgx), uy = fma(jy, cirho, hgy);
+  const double utx = ux - hgx, uty = uy - hgy;
   const double ut2 = fma(uty, uty, utx * utx), g2 = fma(g[1], g[1], g[0] * g[0]);
   const double gu = fma(g[1], uy, g[0] * ux);
   m.u2 = fma(uy, uy, ux * ux);
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_split(const double* __re
     const double ox3 = fma(t.xx, c.O30, fma(t.xy, c.O21, fma(t.yy, c.O12, c.O10)));
     const double oy3 = fma(t.yy, c.O03, c.O01);
     const double odd = fma(t.x, ox3, t.y * oy3);
-    const double ev = fma(hom1, s[r], t.w * even), od = fma(hom1, a[r], t.w * odd);
+    const double ev = fma(hom1, s[r], t.wg * even), od = fma(hom1, a[r], t.wg * odd);
     if (own < n && k < SPLIT_SLOTS) {
       const int i = k < SPLIT_SLOTS - 1 ? 2 * k + 1 : 0;
       fout[i * N + site] = (ev + od) + t.w;
@@ -412,11 +412,13 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_sym(const double* __rest
   jy += jxo;
   // ---- mid-point state (local frame)
   const double rho = 1.0 + m0, irho = 1.0 / rho;
-  const double cirho = L::c * irho;
-  const double ux = fma(0.5, g[0], jx * cirho), uy = fma(0.5, g[1], jy * cirho);
+  const double cirho = L::c * irho, hgx = 0.5 * g[0], hgy = 0.5 * g[1];
+  const double ux = fma(jx, cirho, hgx), uy = fma(jy, cirho, hgy);
+  const double utx = ux - hgx, uty = uy - hgy;
+  const double ut2 = fma(uty, uty, utx * utx), g2 = fma(g[1], g[1], g[0] * g[0]);
   const double gu = fma(g[1], uy, g[0] * ux);
   const double u2 = fma(uy, uy, ux * ux);
-  const double Th = 0.5 * fma(fma(L::c2, k2, -2.0 * m0), irho, gu - u2);
+  const double Th = fma(fma(fma(L::c2, k2, -2.0 * m0), irho, -ut2), 0.5, 0.125 * g2);
   const double om = site_omega<double>(p, rho, 1.0 + Th);
   const double rom = rho * om;
   const double rk = fma(-0.5, rom, rho);
@@ -429,16 +431,15 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_sym(const double* __rest
   {
     const double xx = X * X, xy = X * Y;
     const double b0 = fma(-0.5, u2, fma(-2.0, Th, 1.0));
-    const double hax = 0.5 * (T + xx), T3 = 3.0 * T, T3x = T3 + xx, th2 = 0.5 * Th;
+    const double hT = 0.5 * T, hax = fma(0.5, xx, hT), th2 = 0.5 * Th;
     const double a00 = fma(fma(0.125, u2, Th), u2, fma(Th, Th, fma(-0.5, u2, -Th)));
     c.E00 = fma(rom, a00, FO >= 1 ? fma(om, m0, -rkgu) : om * m0);
-    const double qr = rom * (1.0 / 24.0);
     const double rx = rom * X;
     c.E20 = rom * fma(b0, hax, -(th2 * xx));
     c.E11 = rom * (b0 - Th) * xy;
-    c.E40 = qr * fma(xx, fma(2.0, T3, xx), T3 * T);
+    c.E40 = rom * fma(xx, fma(1.0 / 24.0, xx, 0.25 * T), 0.5 * hT * hT);
     c.E22 = rom * hax * other(hax);
-    c.O30 = (1.0 / 6.0) * rx * T3x;
+    c.O30 = rx * fma(1.0 / 6.0, xx, hT);
     c.E31 = c.O30 * Y;
     if constexpr (FO >= 1) {
       c.E20 = fma(Sx, X, c.E20);
@@ -490,9 +491,10 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_sym(const double* __rest
   const double xa1 = c.E00 + (c.E20 + c.E40), xa2 = fma(4.0, fma(4.0, c.E40, c.E20), c.E00),
                xa3 = fma(9.0, fma(9.0, c.E40, c.E20), c.E00);
   const double za1 = c.O10 + c.O30, za2 = fma(4.0, c.O30, c.O10), za3 = fma(9.0, c.O30, c.O10);
+  constexpr double g9 = collision_w<L>(dir_of(3, 0)), g8 = collision_w<L>(dir_of(2, 2));
   put(ic<0>{}, wk[0], wk[0] * xa1, wk[0] * za1);
   put(ic<1>{}, wk[1], wk[1] * xa2, 2.0 * wk[1] * za2);
-  put(ic<2>{}, wk[2], wk[2] * xa3, 3.0 * wk[2] * za3);
+  put(ic<2>{}, wk[2], g9 * xa3, 3.0 * g9 * za3);
   auto quad = [&](auto K, double w, double A, double xa, double xb, double ya, double za, double wa) {  // (A, +-1)
     constexpr int k = K;
     const double ee = w * (xa + (xb + c.E04)), oo = ya + c.E13, oe = w * A * (za + c.O12), eo = wa + c.O03;
@@ -502,11 +504,12 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_sym(const double* __rest
   quad(ic<3>{}, wk[3], 2.0, xa2, fma(4.0, c.E22, c.E02), fma(4.0, c.E31, c.E11), za2, fma(4.0, c.O21, c.O01));
   quad(ic<5>{}, wk[5], 3.0, xa3, fma(9.0, c.E22, c.E02), fma(9.0, c.E31, c.E11), za3, fma(9.0, c.O21, c.O01));
   {  // (q, +-q)
-    const double ee = wq * fma(qq, fma(qq, (c.E40 + c.E04) + c.E22, c.E20 + c.E02), c.E00);
+    const double gq = role ? g8 : w11;
+    const double ee = gq * fma(qq, fma(qq, (c.E40 + c.E04) + c.E22, c.E20 + c.E02), c.E00);
     const double oo = fma(qq, c.E31 + c.E13, c.E11);
-    const double wqq = wq * q;
+    const double wqq = gq * q;
     const double oe = wqq * fma(qq, c.O30 + c.O12, c.O10), eo = fma(qq, c.O03 + c.O21, c.O01);
-    const double wq2 = wq * qq;
+    const double wq2 = gq * qq;
     put(ic<7>{}, wq, fma(wq2, oo, ee), fma(wqq, eo, oe));
     put(ic<8>{}, wq, fma(-wq2, oo, ee), fma(-wqq, eo, oe));
   }
