@@ -185,11 +185,13 @@ __device__ __forceinline__ void collide2(const unsigned (&h)[L::Q], const float2
 #define LBM_HALF2_BLOCKS 4
 #endif
 
-// Rows of a launch over n layers of the wall axis: with walls and n >= 6 the
-// six rows at the ends take two block indices each, one per half of the
-// block's sites, since they go site by site (and they come first, see
-// wall_rows_first).
-inline int half2_rows(int n, bool walls) { return walls && n >= 6 ? n + 6 : n; }
+// Whether the six rows at the ends of n layers of the wall axis take two block
+// indices each, one per half of the block's sites, since they go site by site
+// (and they come first, see wall_rows_first): with walls, while a launch can
+// have that many rows.
+__host__ __device__ constexpr bool half2_twice(int n, bool walls) { return walls && n >= 6 && n + 6 <= MAX_GRID_YZ; }
+// Rows of a launch.
+inline int half2_rows(int n, bool walls) { return half2_twice(n, walls) ? n + 6 : n; }
 
 // Whether the plain step of an FP16 grid runs two sites per thread.  Needs an
 // even nx (rows then start on a word).  Measured on GB300, microseconds a step
@@ -216,7 +218,7 @@ __global__ void __launch_bounds__(128, LBM_HALF2_BLOCKS)
     k_step_half2(const __half* __restrict__ fin, __half* __restrict__ fout, const StepParams p) {
   constexpr int D = L::D, Q = L::Q;
   const int bx = blockDim.x;
-  const bool twice = p.wall != W_NONE && p.na >= 6;
+  const bool twice = half2_twice(p.na, p.wall != W_NONE);
   const int b = D == 2 ? blockIdx.y : blockIdx.z;
   const int k0 = twice && b < 12 ? b & 1 : 0, k1 = twice && b < 12 ? k0 + 1 : 2;
   const int a = p.a0 + (twice ? wall_rows_first(b < 12 ? b >> 1 : b - 6, p.na, true) : b);

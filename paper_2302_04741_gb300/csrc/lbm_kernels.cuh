@@ -623,6 +623,9 @@ __device__ __forceinline__ int launch_line(int b, int n, bool walls, int reverse
   return b < 3 ? b : (b < 6 ? n - 6 + b : (reverse ? n + 2 - b : b - 3));
 }
 
+// Blocks of a launch along y and along z.
+constexpr int MAX_GRID_YZ = 65535;
+
 // Class of every site of a grid with solid sites, and the list of the fluid
 // sites next to one: pass 0 counts them, pass 1 writes the list.
 template <class L>
