@@ -842,8 +842,9 @@ int lbm_set_solid(lbm_ctx* c, const unsigned char* solid, const double* T_wall) 
     cudaFree(c->wall_sites);
     c->wall_sites = nullptr;
   }
+  c->p.n_wall_sites = (int)n_wall;
+  if (!lbm::wall_list(c->opt.precision, c->N) || !lbm::wall_list_fits(c->D, c->p, c->opt.block_x)) n_wall = 0;
   c->p.n_wall_sites = 0;
-  if (!lbm::wall_list(c->opt.precision, c->N)) n_wall = 0;
   if (n_wall) {
     if (cudaMalloc(&c->wall_sites, sizeof(int) * (size_t)n_wall) != cudaSuccess) {
       cudaGetLastError();

@@ -670,6 +670,10 @@ inline int wall_site_lines(const StepParams& p, int bx) {
   const long long line = (long long)((p.nx + bx - 1) / bx) * (D == 2 ? 1 : p.ny) * bx;
   return (int)((p.n_wall_sites + line - 1) / line);
 }
+// Whether a launch has room for them and the grid.
+inline bool wall_list_fits(int D, const StepParams& p, int bx) {
+  return p.na + (D == 2 ? wall_site_lines<2>(p, bx) : wall_site_lines<3>(p, bx)) <= MAX_GRID_YZ;
+}
 
 // SOLID: the grid has solid sites.  They are skipped; fluid sites next to one take
 // the diffuse-wall pull.

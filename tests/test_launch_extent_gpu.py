@@ -1,10 +1,14 @@
 """Grids as tall as a launch can be (65,535 blocks along y): the step adds no rows to a
 launch that has no room for them."""
+import os
+
 import numpy as np
 import pytest
 
+import oracle
 import paper_2302_04741_gb300 as lbm
-from helpers import workload
+from paper_2302_04741_gb300 import workloads as W
+from helpers import oracle_sim, perm_to_oracle, workload
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -14,6 +18,7 @@ pytestmark = pytest.mark.gpu
 def built():
     from paper_2302_04741_gb300 import build
     build.build()
+    oracle.set_threads(os.cpu_count() or 1)
 
 
 # 65,529 rows leave room for the six rows that are visited twice, 65,530 do not
@@ -35,3 +40,19 @@ def test_fp16_rows_at_walls(ny):
         assert torch.equal(got, want)
     finally:
         lbm.lbm_batch_destroy(b)
+
+
+@pytest.mark.parametrize("lat,shape", [(0, (32, 40000, 1)), (1, (8, 5, 40000))], ids=["32x40000", "8x5x40000"])
+def test_sites_next_to_solids(lat, shape):
+    """As many sites next to solid ones as would take the launch past its last row.  Tolerance
+    per population after two steps: some 40 rounded operations on terms below 0.3 a step,
+    40 x 2 x 0.3 x 2^-53 = 2.7e-15."""
+    N = shape[0] * shape[1] * shape[2]
+    w = workload(lat, shape)
+    w["solid"] = (W.uniform(3, 8, N) < 0.3).astype(np.uint8)
+    w["T_wall"] = 1.0 + 0.1 * (W.uniform(5, 9, N) - 0.5)
+    sim, ref = lbm.Sim(w, block_x=32).init(), oracle_sim(w)
+    sim.step(2)
+    ref.step(2)
+    off = np.abs(sim.populations() - ref.pulled()[perm_to_oracle(lat)])[:, w["solid"] == 0]
+    assert off.max() < 2.7e-15
