@@ -831,19 +831,19 @@ int lbm_set_solid(lbm_ctx* c, const unsigned char* solid, const double* T_wall) 
   LBM_CUDA(c, cudaMemcpy(c->wall_th, th.data(), N * sizeof(double), cudaMemcpyHostToDevice));
   LBM_CUDA(c, cudaMemcpy(c->wall_th_f, thf.data(), N * sizeof(float), cudaMemcpyHostToDevice));
   // the fluid sites next to a solid one: counted, then listed (wall_list)
-  unsigned n_wall = 0;
-  LBM_CUDA(c, cudaMemsetAsync(c->ticket, 0, sizeof(unsigned), c->stream));
-  LBM_CUDA(c, c->ops->classify(c->solid, c->site_class, nullptr, c->ticket, 0, c->p, c->stream));
-  LBM_CUDA(c, cudaMemcpyAsync(&n_wall, c->ticket, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
-  LBM_CUDA(c, cudaMemsetAsync(c->ticket, 0, sizeof(unsigned), c->stream));
+  unsigned count[3] = {};
+  LBM_CUDA(c, cudaMemsetAsync(c->dmax, 0, sizeof count, c->stream));
+  LBM_CUDA(c, c->ops->classify(c->solid, c->site_class, nullptr, c->dmax, 0, c->p, c->stream));
+  LBM_CUDA(c, cudaMemcpyAsync(count, c->dmax, sizeof count, cudaMemcpyDeviceToHost, c->stream));
   LBM_CUDA(c, cudaStreamSynchronize(c->stream));
+  unsigned n_wall = count[0];
   if (c->wall_sites) {  // set a second time before lbm_init
     c->bytes -= sizeof(int) * (size_t)c->p.n_wall_sites;
     cudaFree(c->wall_sites);
     c->wall_sites = nullptr;
   }
   c->p.n_wall_sites = (int)n_wall;
-  if (!lbm::wall_list(c->opt.precision, c->N) || !lbm::wall_list_fits(c->D, c->p, c->opt.block_x)) n_wall = 0;
+  if (!lbm::wall_list(c->opt.precision, c->N, count) || !lbm::wall_list_fits(c->D, c->p, c->opt.block_x)) n_wall = 0;
   c->p.n_wall_sites = 0;
   if (n_wall) {
     if (cudaMalloc(&c->wall_sites, sizeof(int) * (size_t)n_wall) != cudaSuccess) {
@@ -851,8 +851,8 @@ int lbm_set_solid(lbm_ctx* c, const unsigned char* solid, const double* T_wall) 
       return fail(c, LBM_ENOMEM, "device allocation of the wall-site list failed");
     }
     c->bytes += sizeof(int) * (size_t)n_wall;
-    LBM_CUDA(c, c->ops->classify(c->solid, c->site_class, c->wall_sites, c->ticket, 1, c->p, c->stream));
-    LBM_CUDA(c, cudaMemsetAsync(c->ticket, 0, sizeof(unsigned), c->stream));
+    LBM_CUDA(c, cudaMemsetAsync(c->dmax, 0, sizeof count, c->stream));
+    LBM_CUDA(c, c->ops->classify(c->solid, c->site_class, c->wall_sites, c->dmax, 1, c->p, c->stream));
     LBM_CUDA(c, cudaStreamSynchronize(c->stream));
   }
   c->p.site_class = c->site_class;

@@ -49,7 +49,7 @@ struct lbm_ctx {
   unsigned* bad = nullptr;     // bad-site counts per block
   double* dres = nullptr;      // final reduction result (when hres is not mapped)
   unsigned* ticket = nullptr;  // last-block ticket of the conservation pass
-  unsigned* dmax = nullptr;    // FP16 init: max |d| bits per shell
+  unsigned* dmax = nullptr;    // FP16 init: max |d| bits per shell; lbm_set_solid: counts
   double* hres = nullptr;      // pinned host copy of the result
   double* tmp = nullptr;       // (2 + 2D) * N doubles, lazily allocated
   int nblk_cons = 0;

@@ -626,17 +626,21 @@ __device__ __forceinline__ int launch_line(int b, int n, bool walls, int reverse
 // Blocks of a launch along y and along z.
 constexpr int MAX_GRID_YZ = 65535;
 
-// Class of every site of a grid with solid sites, and the list of the fluid
-// sites next to one: pass 0 counts them, pass 1 writes the list.
+// Class of every site of a grid with solid sites, and the list of the fluid sites next
+// to one, a warp for 32 sites of a row as the step has them.  Pass 0: count[0] those
+// sites, count[1] the warps that have one, count[2] the warps that have one and a fluid
+// site away from all solid ones too.  Pass 1: the list, count[0] its length so far.
 template <class L>
 __global__ void __launch_bounds__(256) k_classify(const unsigned char* __restrict__ solid, unsigned char* __restrict__ cls,
                                                   int* __restrict__ list, unsigned* __restrict__ count, int pass,
                                                   const StepParams p) {
-  const int site = blockIdx.x * 256 + threadIdx.x;
-  if (site >= p.N) return;
-  unsigned char c = solid[site] ? 1 : 0;
+  const int per_row = (p.nx + 31) / 32, lane = threadIdx.x & 31;
+  const long long warp = ((long long)blockIdx.x * 256 + threadIdx.x) / 32;
+  if (warp >= (long long)per_row * (p.N / p.nx)) return;
+  const int row = (int)(warp / per_row), x = (int)(warp % per_row) * 32 + lane, site = row * p.nx + x;
+  unsigned char c = x >= p.nx || solid[site] ? 1 : 0;
   if (!c) {
-    const int x = site % p.nx, row = site / p.nx, y = row % p.ny, z = row / p.ny;
+    const int y = row % p.ny, z = row / p.ny;
     static_for<1, L::Q>([&](auto I) {
       constexpr int i = I;
       const int sx = wrap3(x - L::E(i, 0), p.nx), sy = wrap3(y - L::E(i, 1), p.ny);
@@ -644,15 +648,29 @@ __global__ void __launch_bounds__(256) k_classify(const unsigned char* __restric
       if (solid[(sz * p.ny + sy) * p.nx + sx]) c = 2;
     });
   }
-  if (pass == 0) cls[site] = c;
-  if (c == 2) {
-    const unsigned k = atomicAdd(count, 1u);
-    if (pass == 1) list[k] = site;
+  const unsigned wall = __ballot_sync(0xffffffffu, c == 2), plain = __ballot_sync(0xffffffffu, c == 0);
+  if (pass == 0) {
+    if (x < p.nx) cls[site] = c;
+    if (wall && lane < 3 && (lane < 2 || plain)) atomicAdd(count + lane, lane == 0 ? __popc(wall) : 1u);
+  } else if (wall) {
+    unsigned at = 0u;
+    if (lane == 0) at = atomicAdd(count, (unsigned)__popc(wall));
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(wall & ((1u << lane) - 1u));
+    if (c == 2) list[at] = site;
   }
 }
 
-// Whether a grid keeps the list of its wall sites (SOLID_LIST): the FP64 step once it
-// fills the chip.  Below, a step lasts as long as one warp's pull, and a warp of
+// Whether a grid keeps the list of its wall sites (SOLID_LIST), from k_classify's counts: the
+// FP64 step once it fills the chip, where the list saves work.  In place a warp with a wall
+// site takes about twice the time of one without; with the list it takes that for every 32
+// wall sites, and a plain pass for each warp that is left with another site.  So the list
+// pays for a thin wall, and where nearly every fluid site is at one, not for solids scattered
+// so that most warps keep a few sites of both kinds.  GB300, us a step in place -> with the
+// list: 512 x 512 annulus 227 -> 192, 0.4 % of the sites solid 326 -> 271, 5 % 430 -> 531, 30 %
+// 448 -> 341; 80^3 with 0.4 % 964 -> 673, 5 % 1024 -> 1149, 30 % 1031 -> 579, a ball 626 -> 572.
+// (A channel's flat walls, where both sides are equal: 79 -> 64 at 256 x 256 alone, 51 with
+// three grids at once either way.)
+// Below LBM_WALL_LIST_MIN_SITES a step lasts as long as one warp's pull, and a warp of
 // listed sites, whose missing slots differ, runs every slot's wall branch.  GB300,
 // cylinders in FP64, us for 40 steps alone / per grid with three at once, list then in
 // place: 160 x 160 2809 / 1220, 2303 / 1145; 176 x 176 2830 / 1278, 2766 / 1335;
@@ -661,7 +679,9 @@ __global__ void __launch_bounds__(256) k_classify(const unsigned char* __restric
 #ifndef LBM_WALL_LIST_MIN_SITES
 #define LBM_WALL_LIST_MIN_SITES 28672
 #endif
-inline bool wall_list(int precision, long long sites) { return precision == P_FP64 && sites >= LBM_WALL_LIST_MIN_SITES; }
+inline bool wall_list(int precision, long long sites, const unsigned (&count)[3]) {
+  return precision == P_FP64 && sites >= LBM_WALL_LIST_MIN_SITES && count[2] + count[0] / 16.0 <= 2.0 * count[1];
+}
 
 // Lines (y rows in 2-D, z layers in 3-D) that the list of wall sites adds in front
 // of a step's grid of blocks of bx threads.

@@ -28,7 +28,7 @@ struct LatticeOps {
                             const StepParams& p, int nsm, cudaStream_t s);
   int nshell;
   const double* shell_w;
-  // classes of the sites of a grid with solid sites (k_classify)
+  // classes of the sites of a grid with solid sites (k_classify; count: 3 zeroed words)
   cudaError_t (*classify)(const unsigned char* solid, unsigned char* cls, int* list, unsigned* count, int pass,
                           const StepParams& p, cudaStream_t s);
   cudaError_t (*moments)(int P, const void* fin, double* rho, double* u, double* T, double* q,
@@ -215,7 +215,8 @@ struct Ops {
 
   static cudaError_t classify(const unsigned char* solid, unsigned char* cls, int* list, unsigned* count, int pass,
                               const StepParams& p, cudaStream_t s) {
-    k_classify<L><<<(unsigned)(((long long)p.N + 255) / 256), 256, 0, s>>>(solid, cls, list, count, pass, p);
+    const long long warps = (long long)((p.nx + 31) / 32) * (p.N / p.nx);
+    k_classify<L><<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(solid, cls, list, count, pass, p);
     return cudaGetLastError();
   }
 
