@@ -819,10 +819,29 @@ int lbm_set_solid(lbm_ctx* c, const unsigned char* solid, const double* T_wall) 
       thf[k] = (float)th[k];
     }
   }
+  // From here to the end of the uploads the tables are neither the old ones nor the
+  // new: a call that fails in between leaves a grid without solid sites.
+  StepParams& p = c->p;
+  if (c->wall_sites) {  // set a second time before lbm_init
+    c->bytes -= sizeof(int) * (size_t)p.n_wall_sites;
+    cudaFree(c->wall_sites);
+    c->wall_sites = nullptr;
+  }
+  p.solid = p.site_class = nullptr;
+  p.wall_sites = nullptr;
+  p.n_wall_sites = 0;
+  drop_graphs(c);
   if (!c->solid) {
     if (cudaMalloc(&c->solid, N) != cudaSuccess || cudaMalloc(&c->wall_th, N * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&c->wall_th_f, N * sizeof(float)) != cudaSuccess || cudaMalloc(&c->site_class, N) != cudaSuccess) {
       cudaGetLastError();
+      cudaFree(c->solid);
+      cudaFree(c->wall_th);
+      cudaFree(c->wall_th_f);
+      c->solid = nullptr;
+      c->wall_th = nullptr;
+      c->wall_th_f = nullptr;
+      c->site_class = nullptr;
       return fail(c, LBM_ENOMEM, "device allocation of the solid-site tables failed");
     }
     c->bytes += N * (2 + sizeof(double) + sizeof(float));
@@ -833,35 +852,33 @@ int lbm_set_solid(lbm_ctx* c, const unsigned char* solid, const double* T_wall) 
   // the fluid sites next to a solid one: counted, then listed (wall_list)
   unsigned count[3] = {};
   LBM_CUDA(c, cudaMemsetAsync(c->dmax, 0, sizeof count, c->stream));
-  LBM_CUDA(c, c->ops->classify(c->solid, c->site_class, nullptr, c->dmax, 0, c->p, c->stream));
+  LBM_CUDA(c, c->ops->classify(c->solid, c->site_class, nullptr, c->dmax, 0, p, c->stream));
   LBM_CUDA(c, cudaMemcpyAsync(count, c->dmax, sizeof count, cudaMemcpyDeviceToHost, c->stream));
   LBM_CUDA(c, cudaStreamSynchronize(c->stream));
-  unsigned n_wall = count[0];
-  if (c->wall_sites) {  // set a second time before lbm_init
-    c->bytes -= sizeof(int) * (size_t)c->p.n_wall_sites;
-    cudaFree(c->wall_sites);
-    c->wall_sites = nullptr;
-  }
-  c->p.n_wall_sites = (int)n_wall;
-  if (!lbm::wall_list(c->opt.precision, c->N, count) || !lbm::wall_list_fits(c->D, c->p, c->opt.block_x)) n_wall = 0;
-  c->p.n_wall_sites = 0;
-  if (n_wall) {
-    if (cudaMalloc(&c->wall_sites, sizeof(int) * (size_t)n_wall) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(c, LBM_ENOMEM, "device allocation of the wall-site list failed");
+  p.solid = c->solid;
+  p.site_class = c->site_class;
+  p.wall_th = c->wall_th;
+  p.wall_th_f = c->wall_th_f;
+  StepParams listed = p;
+  listed.n_wall_sites = (int)count[0];
+  if (count[0] && lbm::wall_list(c->opt.precision, c->N, count) && lbm::wall_list_fits(c->D, listed, c->opt.block_x)) {
+    int* list = nullptr;
+    if (cudaMalloc(&list, sizeof(int) * (size_t)count[0]) != cudaSuccess) {
+      cudaGetLastError();  // the sites are then stepped in place
+      return LBM_OK;
     }
-    c->bytes += sizeof(int) * (size_t)n_wall;
-    LBM_CUDA(c, cudaMemsetAsync(c->dmax, 0, sizeof count, c->stream));
-    LBM_CUDA(c, c->ops->classify(c->solid, c->site_class, c->wall_sites, c->dmax, 1, c->p, c->stream));
-    LBM_CUDA(c, cudaStreamSynchronize(c->stream));
+    cudaError_t e = cudaMemsetAsync(c->dmax, 0, sizeof count, c->stream);
+    if (e == cudaSuccess) e = c->ops->classify(c->solid, c->site_class, list, c->dmax, 1, p, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) {
+      cudaFree(list);
+      return fail(c, LBM_ECUDA, "wall-site list failed: %s", cudaGetErrorString(e));
+    }
+    c->bytes += sizeof(int) * (size_t)count[0];
+    c->wall_sites = list;
+    p.wall_sites = list;
+    p.n_wall_sites = (int)count[0];
   }
-  c->p.site_class = c->site_class;
-  c->p.wall_sites = c->wall_sites;
-  c->p.n_wall_sites = (int)n_wall;
-  c->p.solid = c->solid;
-  c->p.wall_th = c->wall_th;
-  c->p.wall_th_f = c->wall_th_f;
-  drop_graphs(c);
   return LBM_OK;
 }
 
