@@ -767,9 +767,10 @@ int lbm_init(lbm_ctx* c, const double* rho, const double* u, const double* T) {
     for (int k = 0; k < c->ops->nshell; ++k) {
       float d;
       std::memcpy(&d, &bits[k], sizeof d);
-      mx = std::max(mx, (float)((double)d / c->ops->shell_w[k]));
+      const float r = (float)((double)d / c->ops->shell_w[k]);
+      if (!std::isfinite(r)) return fail(c, LBM_EINVAL, "initial state is not finite");
+      mx = std::max(mx, r);
     }
-    if (!std::isfinite(mx)) return fail(c, LBM_EINVAL, "initial state is not finite");
     // scale s = 2^k with max |d/w| * s in [2^12, 2^13): headroom of 8x below the
     // half-precision maximum for the state to grow into
     int k = 0;

@@ -905,8 +905,7 @@ __global__ void __launch_bounds__(256) k_init_scale(const double* __restrict__ r
   constexpr int D = L::D;
   const int layer = D == 2 ? p.nx : p.nx * p.ny;
   const int end = (p.a0 + p.na) * layer;
-  float mx[L::NSHELL];
-  for (int k = 0; k < L::NSHELL; ++k) mx[k] = 0.f;
+  unsigned mx[L::NSHELL] = {};  // as bits, in which a NaN is above infinity (fmaxf drops it)
   // (long long: site + stride may pass 2^31)
   for (long long s = (long long)p.a0 * layer + blockIdx.x * 256 + threadIdx.x; s < end; s += (long long)gridDim.x * 256) {
     const int site = (int)s;
@@ -916,14 +915,14 @@ __global__ void __launch_bounds__(256) k_init_scale(const double* __restrict__ r
     init_deviations<L, float>(rho, u, T, force_order, p, x, row % p.ny, row / p.ny, site, d);
     static_for<0, L::Q>([&](auto I) {
       constexpr int i = I;
-      mx[L::SH(i)] = fmaxf(mx[L::SH(i)], fabsf(d[i]));
+      mx[L::SH(i)] = max(mx[L::SH(i)], __float_as_uint(fabsf(d[i])));
     });
   }
   __shared__ unsigned sh[L::NSHELL];
   if (threadIdx.x < L::NSHELL) sh[threadIdx.x] = 0u;
   __syncthreads();
   for (int k = 0; k < L::NSHELL; ++k) {
-    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(mx[k]));
+    const unsigned m = __reduce_max_sync(0xffffffffu, mx[k]);
     if ((threadIdx.x & 31) == 0) atomicMax(sh + k, m);
   }
   __syncthreads();
