@@ -31,6 +31,7 @@ struct lbm_batch {
   bool dirty = true;
   int bx = 128, spt = 1, ctas = 0;
   int launch_ctas = 0;  // CTAs of a launch, for the uploaded members (upload)
+  bool walls = false;   // an uploaded member has walls
   int stage = 0;  // 1: halo-staged kernel (FP32-shifted, one site per thread)
   int graph_steps = 0;
   cudaGraphExec_t graph = nullptr;
@@ -89,8 +90,11 @@ int upload(lbm_batch* b) {
   long long tiles = 0;
   const int n = (int)b->members.size();
   size_t bytes = 0;  // the launch's working set: both buffers of every member
-  for (int g = 0; g < n; ++g)
+  bool walls = false;
+  for (int g = 0; g < n; ++g) {
     bytes += 2 * (size_t)b->members[g]->Q * b->members[g]->N * b->members[g]->elem;
+    walls = walls || b->members[g]->p.wall != lbm::W_NONE;
+  }
   const int evict_first = lbm::l2_evict_first_for(bytes, b->device);
   for (int g = 0; g < n; ++g) {
     lbm_ctx* c = b->members[g];
@@ -118,6 +122,8 @@ int upload(lbm_batch* b) {
     drop_graph(b);
     b->launch_ctas = launch;
   }
+  if (walls != b->walls) drop_graph(b);  // the other kernel
+  b->walls = walls;
   b->h_header[2] = (int)((tiles + b->launch_ctas - 1) / b->launch_ctas);
   if (n) BCUDA(b, cudaMemcpyAsync(b->d_grids, b->h_grids, sizeof(lbm::BatchGrid) * n,
                                   cudaMemcpyHostToDevice, b->stream));
@@ -136,7 +142,7 @@ int launch(lbm_batch* b, int k) {
                                        b->launch_ctas, b->bx, b->stream));
     return LBM_OK;
   }
-  BCUDA(b, b->ops->batch_step(b->precision, b->force_order, b->spt, b->d_grids, b->d_prefix,
+  BCUDA(b, b->ops->batch_step(b->precision, b->force_order, b->spt, b->walls, b->d_grids, b->d_prefix,
                               b->d_header, k, b->launch_ctas, b->bx, b->stream));
   return LBM_OK;
 }

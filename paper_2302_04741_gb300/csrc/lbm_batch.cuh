@@ -34,7 +34,14 @@ constexpr int BATCH_STAGED = (int)(offsetof(BatchGrid, p) + offsetof(StepParams,
 
 // header[0] = number of grids, header[1] = number of tiles, header[2] = tiles
 // per CTA (enough that the launch covers them all)
-template <class L, int P, int FO, int SPT>
+// WALLS: a grid of the launch has walls.  A kernel of its own without them, since the code of
+// the wall rows costs the others registers.  How those rows pull hangs on what spills least
+// (80 registers).  GB300, us a step with thermal walls, through a call as before -> here: 12
+// FP32 grids of 64 x 64 x 12 55.5 -> 41.4 (one copy of the code for both walls), 4 of 96^3
+// 201.9 -> 186; in FP16 (inline) 54.8 -> 43.5 and 184 -> 181, bounce-back walls 186 -> 184.
+// D3Q39 in FP16 without walls keeps the call, which no row then takes: with it the compiler
+// schedules the other rows' loads better (4 grids of 96^3 161 -> 156, 24 of 32^3 41.8 -> 40.9).
+template <class L, int P, int FO, int SPT, bool WALLS>
 __global__ void __launch_bounds__(256, min_blocks<L, P>())
     k_step_batch(const BatchGrid* __restrict__ grids, const int* __restrict__ prefix,
                  const int* __restrict__ header, int k) {
@@ -48,13 +55,10 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
   const int bx = blockDim.x, TW = bx * SPT;
   int gcur = -1;
   // A CTA takes a run of consecutive tiles: they share the grid, its staged
-  // parameters and the search for it but at a grid's end.  Rows at a wall pull
-  // through a call: their code, inline, made the loop spill (132 B on D3Q39), but for
-  // D2Q37 in FP32 (8 B), whose wall rows it would only delay (cells with two walls
-  // 94.5 us a step, 98.0 with the call).  GB300, against tiles gridDim.x apart, us a
-  // step: 64 ragged D2Q37 grids FP32 273 -> 252, FP16 241 -> 213; 24 D3Q39 boxes FP32
-  // 341 -> 333, FP16 302 -> 284.  The bound is the traffic (92 % of the copy rate on
-  // the FP32 D2Q37 mix).
+  // parameters and the search for it but at a grid's end.  GB300, against tiles
+  // gridDim.x apart, us a step: 64 ragged D2Q37 grids FP32 273 -> 252, FP16 241 -> 213;
+  // 24 D3Q39 boxes FP32 341 -> 333, FP16 302 -> 284.  The bound is the traffic (92 % of
+  // the copy rate on the FP32 D2Q37 mix).
   const int run = __ldg(header + 2);
   int next = 0, lo = 0;  // first tile of the next grid; this grid
   for (int t = blockIdx.x * run, t1 = min(t + run, ntiles); t < t1; ++t) {
@@ -91,7 +95,7 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
       // one row, wrap around no axis in x and touch no wall
       const int x0 = site0 % p.nx, r0 = site0 / p.nx;
       const int a0 = L::D == 2 ? r0 % p.ny : r0 / p.ny;
-      const bool near0 = p.wall != W_NONE && (a0 < 3 || a0 >= nA - 3);
+      const bool near0 = WALLS && near_wall(p, a0, nA);
       const bool interior = !near0 && x0 >= 3 && x0 + 31 <= p.nx - 4;
       if (site >= p.N) continue;
       const int x = site % p.nx, row = site / p.nx;
@@ -99,8 +103,9 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
       constexpr bool SC = scaled_step<P, FO>();
       R d[L::Q];
       if (interior) pull_interior<L, P, R, LD_RO, SC ? IN_SCALED : IN_DEV>(fin + site, p, y, z, d);
-      else if (!near_wall(p, L::D == 2 ? y : z, nA)) pull_stored<L, P, R, LD_RO, SC ? IN_SCALED : IN_DEV>(fin, p, x, y, z, d);
-      else if (L::D == 2 && P == P_FP32S) pull<L, P, R, LD_RO, SC>(fin, p, x, y, z, d);
+      else if constexpr (WALLS) pull<L, P, R, LD_RO, SC, L::D == 3 && P == P_FP32S>(fin, p, x, y, z, d);
+      else if constexpr (!(L::D == 3 && P == P_FP16S)) pull_stored<L, P, R, LD_RO, SC ? IN_SCALED : IN_DEV>(fin, p, x, y, z, d);
+      else if (!near_wall(p, z, nA)) pull_stored<L, P, R, LD_RO, SC ? IN_SCALED : IN_DEV>(fin, p, x, y, z, d);
       else {
         R w[L::Q];
         pull_call<L, P, LD_RO, SC>(fin, p, x, y, z, w);

@@ -27,27 +27,29 @@ enum Wall { W_NONE = 0, W_BOUNCE = 1, W_THERMAL = 2 };
 enum GKind { G_UNIFORM = 0, G_SINE = 1, G_FIELD = 2 };
 
 // Everything a step kernel needs, passed by value (constant bank).  First what every block
-// of a step in float reads: with these fields together, small grids
-// that are stepped at once in streams of their own (each launch finds its parameters cold in
-// the constant caches) take 5 to 15 % less time than with the wall tables in between: FP32,
-// us a step and grid, 32 grids of 256 x 256 3.61 -> 3.09, of 256 x 128 1.74 -> 1.53, of 40^3
-// 4.48 -> 4.09; one 256 x 256 grid alone 4.73 -> 4.71.
+// of a step in float reads: with these fields together, small grids that are stepped at once
+// in streams of their own (each launch finds its parameters cold in the constant caches) take
+// 5 to 15 % less time than with the wall tables in between: FP32, us a step and grid, 32 grids
+// of 256 x 256 3.61 -> 3.08, of 256 x 128 1.74 -> 1.53, of 40^3 4.48 -> 4.10; one 256 x 256
+// grid alone 4.73 -> 4.73.  (The order among them moves the registers that the batch kernels,
+// at their cap, spill: of eight orders this one spills least.)
 struct StepParams {
+  // float copies for the float kernels (no FP64 conversion on their path)
+  float omega_f;
+  float mu_f;
+  float g0_f[3];
+  int gkind;         // GKind
+  const float* gtab_f;  // float copy of gtab (same layout)
   int nx, ny, nz;    // nz = 1 on D2Q37
   int N;             // sites (< 2^31)
   int wall;          // Wall, on the last axis (y for D = 2, z for D = 3)
-  int gkind;         // GKind
-  int gaxis;         // G_SINE: axis of the wave
   // layers of the last axis the per-site kernels visit: a0 .. a0 + na - 1
   // (the whole axis, a0 = 0 and na = n_axis, except on a slab context, whose
   // buffer also holds the ghost layers of its neighbours)
   int a0, na;
   int l2_evict_first;  // 1: population loads are evict-first in L2 (see ld_pop_policy)
   int reverse;         // 1: the launch visits the lines of the grid in descending order (launch_line)
-  // float copies for the float kernels (no FP64 conversion on their path)
-  float omega_f;
-  float mu_f;
-  float g0_f[3];
+  int gaxis;         // G_SINE: axis of the wave
   float h_scale;      // FP16 codec scale s and 1/s
   float h_inv_scale;
   // lanes per site of the FP64 step on a small D2Q37 grid (lbm_split.cuh), 0: one
@@ -58,7 +60,6 @@ struct StepParams {
   double mu;          // > 0: constant dynamic viscosity, 1/omega = mu/(rho theta) + 1/2 per site
   double g0[3];      // G_UNIFORM / G_SINE amplitude
   const double* gtab;  // G_SINE: sin(2 pi k / n_axis), k < n_axis; G_FIELD: D*N field
-  const float* gtab_f;  // float copy of gtab (same layout)
   // solid sites (staircase walls, fully periodic grids): flag per site and
   // wall temperature minus 1 per site (read at solid sites only); nullptr
   // when the grid has none

@@ -119,7 +119,8 @@ __device__ __forceinline__ RR add_deviation(RR sum, typename Codec<P>::T v, cons
 // Pull of a site in one of the three rows next to the wall on side SIDE: slots
 // whose source lies beyond it follow the wall rule.  The side is a template
 // parameter: the populations that leave the column through the wall (26 on
-// D2Q37) are then a fixed list, loaded without a predicate each.
+// D2Q37) are then a fixed list, loaded without a predicate each.  SIDE -1: either
+// side, known at run time, for a kernel that has no registers for both.
 template <class L, int P, class RR, int LD, bool SC, int SIDE>
 __device__ __forceinline__ void pull_near(const typename Codec<P>::T* __restrict__ fin, const StepParams& p, int x, int y,
                                           int z, int a, int nA, const int (&xs)[7], const int (&ys)[7],
@@ -128,6 +129,7 @@ __device__ __forceinline__ void pull_near(const typename Codec<P>::T* __restrict
   constexpr int D = L::D, Q = L::Q;
   const int nx = p.nx, ny = p.ny;
   const size_t N = (size_t)p.N;
+  const int side = SIDE < 0 ? (a < 3 ? 0 : 1) : SIDE;
   const int colbase = D == 2 ? x : (y * nx + x);     // site of the column at wall coord 0
   const int lineA = D == 2 ? nx : nx * ny;           // stride along the wall axis
   RR rm1 = RR(0);                                    // rho_w - 1 of the thermal wall
@@ -135,31 +137,33 @@ __device__ __forceinline__ void pull_near(const typename Codec<P>::T* __restrict
     RR sum = RR(0);
     static_for<0, 3>([&](auto ROW) {
       constexpr int r = ROW;
-      const int row = SIDE == 0 ? r : nA - 1 - r;
+      const int row = side == 0 ? r : nA - 1 - r;
       static_for<0, Q>([&](auto J) {
         constexpr int j = J;
         constexpr int eA = L::E(j, D - 1);
-        if constexpr (SIDE == 0 ? eA < 0 && r + eA < 0 : eA > 0 && r - eA < 0)
-          sum = add_deviation<L, P, j, r>(sum, ldpop<C, LD>(fin + j * N + colbase + row * lineA, p), p);
+        if constexpr ((SIDE != 1 && r + eA < 0) || (SIDE != 0 && r - eA < 0)) {
+          if (SIDE >= 0 || (side == 0 ? eA < 0 : eA > 0))
+            sum = add_deviation<L, P, j, r>(sum, ldpop<C, LD>(fin + j * N + colbase + row * lineA, p), p);
+        }
       });
     });
-    rm1 = (ParamsOf<RR>::wallA(p, SIDE) + sum) * ParamsOf<RR>::wall_inv_den(p, SIDE);
+    rm1 = (ParamsOf<RR>::wallA(p, side) + sum) * ParamsOf<RR>::wall_inv_den(p, side);
   }
   static_for<0, Q>([&](auto I) {
     constexpr int i = I;
     constexpr int ex = L::E(i, 0), ey = L::E(i, 1), ez = L::E(i, 2);
     constexpr int eA = L::E(i, D - 1);
     const int sA = a - eA;
-    if ((SIDE == 0 ? eA <= 0 : eA >= 0) || (SIDE == 0 ? sA >= 0 : sA < nA)) {
+    if ((SIDE == 0 && eA <= 0) || (SIDE == 1 && eA >= 0) || (side == 0 ? sA >= 0 : sA < nA)) {
       const int off = zs[ez + 3] + ys[ey + 3] + xs[ex + 3];
       d[i] = RR(step_in<L, P, i, SC>(ldpop<C, LD>(fin + i * N + off, p), p));
     } else if (p.wall == W_BOUNCE) {
       // d_i = d_io and w_i = w_io: the scaled values agree as well
       constexpr int io = opposite<i>();
-      const int mA = SIDE == 0 ? eA - 1 - a : 2 * nA - 1 - sA;
+      const int mA = side == 0 ? eA - 1 - a : 2 * nA - 1 - sA;
       d[i] = RR(step_in<L, P, io, SC>(ldpop<C, LD>(fin + io * N + colbase + mA * lineA, p), p));
     } else {
-      d[i] = step_from_dev<i, SC>(fma(rm1, ParamsOf<RR>::fw(p, SIDE, i), ParamsOf<RR>::fwd(p, SIDE, i)), p);
+      d[i] = step_from_dev<i, SC>(fma(rm1, ParamsOf<RR>::fw(p, side, i), ParamsOf<RR>::fwd(p, side, i)), p);
     }
   });
 }
@@ -167,7 +171,8 @@ __device__ __forceinline__ void pull_near(const typename Codec<P>::T* __restrict
 // Pull of all Q populations of site (x, y, z) with the boundary rules, decoded
 // to deviations in type RR (SC: the scaled values of an FP16-scaled step, see
 // scaled_step).  The wall axis is the last axis (y in 2-D, z in 3-D).
-template <class L, int P, class RR, int LD = LD_HINT, bool SC = false>
+// BOTH: one copy of the wall rows' code for both sides.
+template <class L, int P, class RR, int LD = LD_HINT, bool SC = false, bool BOTH = false>
 __device__ __forceinline__ void pull(const typename Codec<P>::T* __restrict__ fin,
                                      const StepParams& p, int x, int y, int z, RR (&d)[L::Q]) {
   using C = Codec<P>;
@@ -193,7 +198,8 @@ __device__ __forceinline__ void pull(const typename Codec<P>::T* __restrict__ fi
     return;
   }
   // a row next to a wall (block-uniform side)
-  if (a < 3) pull_near<L, P, RR, LD, SC, 0>(fin, p, x, y, z, a, nA, xs, ys, zs, d);
+  if constexpr (BOTH) pull_near<L, P, RR, LD, SC, -1>(fin, p, x, y, z, a, nA, xs, ys, zs, d);
+  else if (a < 3) pull_near<L, P, RR, LD, SC, 0>(fin, p, x, y, z, a, nA, xs, ys, zs, d);
   else pull_near<L, P, RR, LD, SC, 1>(fin, p, x, y, z, a, nA, xs, ys, zs, d);
 }
 

@@ -53,7 +53,8 @@ struct LatticeOps {
                             int bx, cudaStream_t s);
   // batch step (FP32-shifted and FP16-scaled storage; SPT 1 or 2)
   cudaError_t (*batch_occupancy)(int P, int FO, int spt, int bx, int* blocks_per_sm);
-  cudaError_t (*batch_step)(int P, int FO, int spt, const BatchGrid* grids, const int* prefix,
+  // walls: whether a member has any
+  cudaError_t (*batch_step)(int P, int FO, int spt, bool walls, const BatchGrid* grids, const int* prefix,
                             const int* header, int k, int grid, int bx, cudaStream_t s);
   // halo-staged batch step (FP32-shifted storage, one site per thread)
   cudaError_t (*batch_staged_occupancy)(int FO, int bx, int* blocks_per_sm);
@@ -323,7 +324,7 @@ struct Ops {
 
   template <int PP, int FF, int SS>
   static cudaError_t batch_occ_one(int bx, int* bps) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, k_step_batch<L, PP, FF, SS>, bx, 0);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, k_step_batch<L, PP, FF, SS, true>, bx, 0);
   }
 
   static cudaError_t batch_occupancy(int P, int FO, int spt, int bx, int* bps) {
@@ -335,11 +336,12 @@ struct Ops {
     return cudaErrorInvalidValue;
   }
 
-  static cudaError_t batch_step(int P, int FO, int spt, const BatchGrid* grids, const int* prefix,
+  static cudaError_t batch_step(int P, int FO, int spt, bool walls, const BatchGrid* grids, const int* prefix,
                                 const int* header, int k, int grid, int bx, cudaStream_t s) {
 #define LBM_BSTEP(PP, FF, SS)                                                               \
   if (P == PP && FO == FF && spt == SS) {                                                    \
-    k_step_batch<L, PP, FF, SS><<<grid, bx, 0, s>>>(grids, prefix, header, k);                \
+    if (walls) k_step_batch<L, PP, FF, SS, true><<<grid, bx, 0, s>>>(grids, prefix, header, k); \
+    else k_step_batch<L, PP, FF, SS, false><<<grid, bx, 0, s>>>(grids, prefix, header, k);   \
     return cudaGetLastError();                                                              \
   }
     LBM_BSTEP(1, 0, 1) LBM_BSTEP(1, 1, 1) LBM_BSTEP(1, 2, 1) LBM_BSTEP(1, 0, 2) LBM_BSTEP(1, 1, 2) LBM_BSTEP(1, 2, 2)
