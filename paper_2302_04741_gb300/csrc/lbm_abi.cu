@@ -580,7 +580,7 @@ int create_impl(lbm_lattice lat, int nx, int ny, int nz, double tau, const lbm_g
     int nsm = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device);
     c->nsm = nsm;
-    if (D == 2 && o.precision == LBM_FP64) p.split = lbm::split_lanes(N, nsm);
+    if (D == 2 && o.precision == LBM_FP64) p.split = lbm::split_lanes(nx, N, nsm);
     const long long tiles = (long long)((nx + 127) / 128) * (D == 2 ? na : (long long)ny * na);
     c->nblk_cons = (int)std::min<long long>(tiles, (long long)LBM_CONSERVED_BLOCKS * (nsm > 0 ? nsm : 1));
   }

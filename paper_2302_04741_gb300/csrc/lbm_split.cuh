@@ -14,14 +14,17 @@
 //   k_step_sym: 2 lanes, which exploit that the velocity set maps onto itself
 //     when x and y are swapped (see there): some 265 operations a lane.
 // GB300, microseconds a step (20-step graphs), one thread per site -> here:
-// 3 x 150 with thermal walls 30.0 -> 10.1, 24 x 24 22.6 -> 9.0, 64 x 64 22.7 ->
+// 3 x 150 with thermal walls 30.0 -> 10.1, 24 x 24 22.6 -> 11.4, 64 x 64 22.7 ->
 // 11.6 (17.2 with lbm_poly.cuh alone), with walls 30.0 -> 13.6, 96 x 96 22.8 ->
 // 12.6.  The lanes multiply the FP64 work of a site (4.0 and 1.2 times), which
-// counts when many small grids are stepped in streams of their own; so 8 lanes
+// counts when many small grids are stepped in streams of their own.  So 8 lanes
 // are taken only up to one warp per multiprocessor (3 x 150: 16 lanes take 9.5
 // us alone, but 21.2 for each step of eight grids at once where 8 lanes take
-// 14.0 and one thread 37), 2 lanes up to one warp per sub-partition (eight
-// 64 x 64 at once: 40.9 -> 34.1).
+// 14.0 and one thread 37), and for rows of 12 sites at most, which leave most of
+// a one-thread warp idle anyway: us a step and grid, 64 grids at once, one thread
+// with the collision pair by pair -> 8 lanes, 12 x 50 1.85 -> 1.73, but 16 x 38 1.42 ->
+// 1.75 and 32 x 19 0.76 -> 1.74 (2 lanes 0.61).  2 lanes up to one warp per
+// sub-partition (eight 64 x 64 at once: 40.9 -> 34.1).
 #pragma once
 
 #include "lbm_kernels.cuh"
@@ -75,8 +78,8 @@ static __device__ const SplitTable split_table = make_split_table();
 
 // Lanes per site of a grid of `sites` sites on nsm multiprocessors; 0: one
 // thread per site.
-inline int split_lanes(long long sites, int nsm) {
-  if (sites * 8 <= 32LL * nsm) return 8;        // at most one warp per multiprocessor
+inline int split_lanes(int nx, long long sites, int nsm) {
+  if (nx <= 12 && sites * 8 <= 32LL * nsm) return 8;  // at most one warp per multiprocessor
   if (sites * 2 <= 32LL * 4 * nsm) return 2;    // at most one warp per sub-partition
   return 0;
 }
