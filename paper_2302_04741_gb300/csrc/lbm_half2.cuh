@@ -196,21 +196,25 @@ inline int half2_rows(int n, bool walls) { return half2_twice(n, walls) ? n + 6 
 // Whether the plain step of an FP16 grid runs two sites per thread.  Needs an
 // even nx (rows then start on a word).  Measured on GB300, microseconds a step
 // (one site per thread -> two): 512 x 512 x 256 2860 -> 2178, 256^2 x 128 380 ->
-// 299, 64^3 11.3 -> 7.3, 1024 x 512 18.7 -> 15.1, 4096 x 2048 311 -> 244,
-// 256 x 128 11.4 -> 10.7.  Not taken where a warp of pairs is poorly filled, so
+// 299, 1024 x 512 18.7 -> 15.1, 4096 x 2048 311 -> 244, 512 x 192 5.6 -> 5.4, 256 x 256
+// 4.49 -> 4.45 (eight at once 2.25 -> 1.84 each), 64^3 11.3 -> 7.3, 64 x 32 x 16 3.70 -> 3.67
+// (1.33 -> 0.95).  Not taken where a warp of pairs is poorly filled, so
 // that a row needs nearly as many warps as of single sites (96^3, 3 against 2 a
 // row: 33.7 -> 34.5; 130 columns, 5 against 3: 32.8 -> 28.0), nor on grids so
-// small that a thread's own latency counts (128 x 64: 2.6 -> 3.1).
+// small that a thread's own latency counts, alone (512 x 96 4.0 -> 4.4, 256 x 192 3.95 -> 4.4,
+// 128 x 128 3.1 -> 3.45, 64 x 16 x 16 3.25 -> 3.5) or with walls (256 x 192 6.1 -> 6.5).
+template <int D>
 inline bool half2_serves(const StepParams& p) {
   const int single = (p.nx + 31) / 32, pairs = (p.nx + 63) / 64;
-  return p.nx % 2 == 0 && 5 * single >= 8 * pairs && p.N >= 16384;
+  return p.nx % 2 == 0 && 5 * single >= 8 * pairs && p.N >= (D == 2 ? 65536 : 32768);
 }
 
-// Threads per block: the caller's choice up to 128, no more warps than a row
-// has pairs for.
+// Threads per block: the caller's choice up to 128, the warps that a row has
+// pairs for shared evenly between its blocks (320 columns: two blocks of 96).
 inline int half2_block(int nx, int bx) {
-  const int row = ((nx + 1) / 2 + 31) / 32 * 32;
-  return bx < 128 ? (bx < row ? bx : row) : (row < 128 ? row : 128);
+  const int warps = ((nx + 1) / 2 + 31) / 32, most = (bx < 128 ? bx : 128) / 32;
+  const int blocks = (warps + most - 1) / most;
+  return (warps + blocks - 1) / blocks * 32;
 }
 
 template <class L, int FO>

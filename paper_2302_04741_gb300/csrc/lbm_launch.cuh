@@ -169,7 +169,7 @@ struct Ops {
         return e != cudaSuccess ? e : cudaGetLastError();
       }
     }
-    if (P == P_FP16S && FO <= 2 && half2_serves(p)) {
+    if (P == P_FP16S && FO <= 2 && half2_serves<L::D>(p)) {
       const int b = half2_block(p.nx, bx);
       cfg.blockDim = dim3(b);
       cfg.gridDim = row_grid<L::D>(p, 2 * b);

@@ -26,3 +26,11 @@ def kernel(L, lat, shape, **options):
                                         ((64, 153, 1), "k_stepINS_5D2Q37ELi0E")])
 def test_lanes_of_the_fp64_step(fake, shape, name):  # noqa: F811
     assert name in kernel(fake, lbm.LBM_D2Q37, shape)
+
+
+# two sites a thread: even rows, grids large enough that a thread's latency does not count
+@pytest.mark.parametrize("lat,shape,two", [(0, (512, 128, 1), True), (0, (510, 128, 1), False), (0, (513, 128, 1), False),
+                                           (0, (256, 192, 1), False), (1, (64, 32, 16), True), (1, (64, 31, 16), False)])
+def test_sites_per_thread_of_the_fp16_step(fake, lat, shape, two):  # noqa: F811
+    name = kernel(fake, lat, shape, precision=lbm.LBM_FP16_SCALED)
+    assert ("k_step_half2" in name) == two
