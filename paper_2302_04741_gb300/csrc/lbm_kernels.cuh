@@ -741,10 +741,14 @@ __global__ void __launch_bounds__(256, min_blocks<L, P>())
   }
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= p.nx) return;
-  const bool walls = p.wall != W_NONE;
-  const int y = L::D == 2 ? p.a0 + launch_line(blockIdx.y - lines, p.na, walls, p.reverse)
-                          : (p.reverse ? p.ny - 1 - (int)blockIdx.y : (int)blockIdx.y);
-  const int z = L::D == 3 ? p.a0 + launch_line(blockIdx.z - lines, p.na, walls, p.reverse) : 0;
+  // (a grid with solid sites has no walls, and visits its lines in ascending order: the
+  // other direction cost FP32 grids of 100 x 100 to 512 x 512 up to a fifth of a step, a
+  // channel of 192 x 192 between solid rows 8.9 -> 11.0 us)
+  const int reverse = SOLID == SOLID_NONE ? p.reverse : 0;
+  const bool walls = SOLID == SOLID_NONE && p.wall != W_NONE;
+  const int y = L::D == 2 ? p.a0 + launch_line(blockIdx.y - lines, p.na, walls, reverse)
+                          : (reverse ? p.ny - 1 - (int)blockIdx.y : (int)blockIdx.y);
+  const int z = L::D == 3 ? p.a0 + launch_line(blockIdx.z - lines, p.na, walls, reverse) : 0;
   const int site = (z * p.ny + y) * p.nx + x;
   if constexpr (SOLID == SOLID_LIST) {
     if (__ldg(p.site_class + site)) return;
