@@ -547,33 +547,6 @@ __device__ __forceinline__ RawMoments<L, R> raw_moments_scaled(const R (&h)[L::Q
   return r;
 }
 
-// From the deviations of the pulled distribution.
-template <class L, class R>
-__device__ __forceinline__ void midpoint_state(const R (&d)[L::Q], const R (&g)[3], MidState<L, R>& m) {
-  constexpr int D = L::D;
-  const RawMoments<L, R> r = raw_moments<L, R>(d);
-  const R drho = r.drho;
-  const R rho = R(1) + drho;
-  const R irho = R(1) / rho;
-  const R ut0 = mul_c<L, R>(r.j[0] * irho), ut1 = mul_c<L, R>(r.j[1] * irho),
-          ut2 = mul_c<L, R>(r.j[2] * irho);
-  const R ut_sq = ut0 * ut0 + ut1 * ut1 + ut2 * ut2;
-  const R g2 = g[0] * g[0] + g[1] * g[1] + g[2] * g[2];
-  m.drho = drho;
-  m.rho = rho;
-  m.u[0] = ut0 + R(0.5) * g[0];
-  m.u[1] = ut1 + R(0.5) * g[1];
-  m.u[2] = ut2 + R(0.5) * g[2];
-  m.theta_m1 = ((mul_c2<L, R>(r.k2) - R(D) * drho) * irho - ut_sq) * R(1.0 / D) + g2 * R(0.25 / D);
-  m.u2 = m.u[0] * m.u[0] + m.u[1] * m.u[1] + m.u[2] * m.u[2];
-  m.gu = g[0] * m.u[0] + g[1] * m.u[1] + g[2] * m.u[2];
-  for (int a = 0; a < 3; ++a) {
-    m.cu[a] = mul_c<L, R>(m.u[a]);
-    m.cg[a] = mul_c<L, R>(g[a]);
-  }
-  prepare_shells<L, R>(m);
-}
-
 // From given physical fields (initialisation): drho = rho - 1 and
 // theta_m1 = T - 1 are formed in double by the caller, so that the small
 // deviations keep their precision when R is float.
