@@ -3,7 +3,7 @@
 // GB300 executes FP64 instructions at about 1/73 of the FP32 rate (measured:
 // DFMA and DADD 0.53 T/s, FFMA 38.8 T/s), and its double <-> float
 // conversion instructions run at the FP64 rate too.  The FP64 step (FP64
-// storage, some 440 FP64 operations per site) is therefore bound by the
+// storage, some 420 FP64 operations per site) is therefore bound by the
 // FP64 units at about a tenth of its HBM roofline.  A value held as an
 // unevaluated sum hi + lo of two floats (|lo| <= ulp(hi)) carries about 48
 // significant bits, and its arithmetic -- Dekker's and Knuth's error-free

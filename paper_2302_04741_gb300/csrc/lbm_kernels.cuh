@@ -705,7 +705,7 @@ inline bool wall_list_fits(int D, const StepParams& p, int bx) {
 // the diffuse-wall pull.
 //   SOLID_LIST (wall_list): those sites in blocks of their own, the first of the
 //   launch.  Left among the others, a warp with one such site ran the wall's FP64
-//   operations for all 37 directions, 470 beside the 440 of a plain site, and every
+//   operations for all 37 directions, 470 beside the 420 of a plain site, and every
 //   site read 37 flags.  256 x 256 cylinders FP64, 20 steps and read-out 1.37 -> 1.03 ms.
 //   SOLID_PLACE: among the others, in FP64 only in the warps that have such a site
 //   (146 x 146 cylinders, 40 steps and read-out 2.32 -> 1.87 ms, every site before).

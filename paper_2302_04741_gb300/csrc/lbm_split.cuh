@@ -3,11 +3,11 @@
 // What bounds the one-thread-per-site step on a small grid: a warp's FP64
 // instruction takes 64 cycles on its sub-partition (19 when all four of an SM
 // share the unit) whatever the number of active lanes, dependent or not, so a
-// grid with fewer warps than sub-partitions takes some 440 x 64 cycles a step
+// grid with fewer warps than sub-partitions takes some 420 x 64 cycles a step
 // however small it is.  So several lanes share a site:
 //   k_step_split: 8 lanes; lane g takes the direction pairs g, g + 8, g + 16, its
 //     partial moments are summed by shuffles, every lane forms the site's
-//     coefficients and stores its own pairs: some 215 operations a lane.  The
+//     coefficients and stores its own pairs: some 200 operations a lane.  The
 //     pairs of different lanes run the same instructions, so their directions
 //     are data: small integers unpacked from immediates for the addresses,
 //     doubles from a table.
@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_step_split(const double* __re
 //   (1, 0) (2, 0) (3, 0) (2, +-1) (3, +-1) (q, +-q), q = 1 in lane 0, 2 in lane 1,
 // which together are all eighteen; lane 0 adds the rest particle.  Of the
 // coefficients a lane forms those of its local x and gets those of y from its
-// partner.  Some 265 FP64 operations a lane against 440 in one thread, so a
+// partner.  Some 265 FP64 operations a lane against 420 in one thread, so a
 // grid of few warps takes 0.6 of the time, for 1.2 times the FP64 work.
 struct PairPath {  // population indexes and vector of a local pair's first member in global terms
   int ip, im, ex, ey;
